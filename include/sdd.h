@@ -234,7 +234,10 @@ sdd_status sdd_get_stats(const sdd_problem* p, sdd_stats* out);
  *                       single problem.
  *   blocks_per_sm     : 1 .. max_blocks_per_sm, the register limit of the kernel (read-only
  *                       field, filled by the get calls; ignored by the set calls).
- *   paths_per_task    : 1024, 2048 (the default) or 4096.
+ *   paths_per_task    : 1024, 2048 (the default) or 4096.  A problem whose tasks of that size
+ *                       would leave most warps idle runs finer ones of its own (a power of two,
+ *                       at least 32, fixed by its parameters), compensated sums and FP32 paths of
+ *                       SDD_FORM_DIV on a Dirichlet domain excepted.
  * What does and does not change results: threads_per_block and blocks_per_sm never do (every
  * warp runs whole tasks of fixed paths, and the sums are reduced task by task in a fixed order).
  * paths_per_task groups a node's paths differently for the estimator sums (per lane, per task,

@@ -260,6 +260,7 @@ McParams<T> mc_params(const sdd_problem* p)
     P.node_of = p->node_of; P.p_begin = p->p_begin; P.p_count = p->p_count;
     P.task_off = p->task_off; P.n_active = p->n_active; P.task_counter = p->task_counter;
     P.slots = p->slots;
+    P.task_len = p->task_len;
     P.task_paths = p->task_paths;
     return P;
 }
@@ -270,10 +271,12 @@ sdd_status launch_mc_round(sdd_problem* p, bool debug, double* dval, int32_t* ds
     if (p->fp64) {
         McParams<double> P = mc_params<double>(p);
         P.dbg_val = dval; P.dbg_steps = dsteps; P.dbg_side = dside; P.dbg_p0 = dp0; P.dbg_n = dn;
+        if (debug) P.task_len = nullptr;  // the debug plan is cut into tasks of task_paths
         SDD_CK(launch_mc<double>(P, p->acc_mode, debug, false, p->mc_grid, p->stream));
     } else {
         McParams<float> P = mc_params<float>(p);
         P.dbg_val = dval; P.dbg_steps = dsteps; P.dbg_side = dside; P.dbg_p0 = dp0; P.dbg_n = dn;
+        if (debug) P.task_len = nullptr;  // the debug plan is cut into tasks of task_paths
         SDD_CK(launch_mc<float>(P, p->acc_mode, debug, false, p->mc_grid, p->stream));
     }
     return SDD_OK;
@@ -326,6 +329,8 @@ sdd_status run_mc(sdd_problem* p, int lo = 0, int hi = -1)
     PP.p_begin = p->p_begin; PP.p_count = p->p_count; PP.task_off = p->task_off;
     PP.n_active = p->n_active; PP.task_counter = p->task_counter;
     PP.task_paths = p->task_paths;
+    PP.fill = p->fill();
+    PP.task_len = p->task_len;
     ReduceParams RP{};
     RP.node_of = p->node_of; RP.p_count = p->p_count; RP.task_off = p->task_off;
     RP.n_active = p->n_active; RP.slots = p->slots; RP.shift = p->shift; RP.acc = p->acc;
@@ -496,7 +501,7 @@ void problem_arrays(sdd_problem* p, bool with_mc, F&& f)
         f((void**)&p->acc, (M + 1) * 32); f((void**)&p->n_done, (M + 1) * 8); f((void**)&p->steps, (M + 1) * 8);
         f((void**)&p->paths_run, (M + 1) * 8); f((void**)&p->next_total, (M + 1) * 8);
         f((void**)&p->node_of, (M + 1) * 4); f((void**)&p->p_begin, (M + 1) * 8); f((void**)&p->p_count, (M + 1) * 8);
-        f((void**)&p->task_off, (M + 2) * 8); f((void**)&p->n_active, 16); f((void**)&p->task_counter, 16);
+        f((void**)&p->task_off, (M + 2) * 8); f((void**)&p->task_len, (M + 1) * 4); f((void**)&p->n_active, 16); f((void**)&p->task_counter, 16);
         f((void**)&p->slots, (size_t)p->slot_cap * sizeof(TaskSlot));
         f((void**)&p->est, (M + 1) * 16); f((void**)&p->se, (M + 1) * 16);
     }
@@ -1007,6 +1012,9 @@ sdd_status sdd_tune(sdd_problem* p, int32_t tune_paths_per_task, sdd_mc_config* 
             // paths of the round at this task size (a round gives a node at most 256 tasks)
             const int64_t round = n0 < (int64_t)kTasksPerRound * T ? n0 : (int64_t)kTasksPerRound * T;
             PP.task_paths = T;
+            PP.task_len = p->task_len;
+            PP.fill = fill_task_paths(p->M, n0, T, p->fp64, p->acc_mode,
+                                      p->prm.form, p->prm.periodic, p->prm.substeps);
             for (int bps = 1; bps <= p->mc_max_blocks_per_sm && ce == cudaSuccess; ++bps) {
                 float ms_min = 0.f;
                 for (int rep = 0; rep < 2 && ce == cudaSuccess; ++rep) {

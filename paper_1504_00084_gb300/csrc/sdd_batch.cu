@@ -53,11 +53,13 @@ struct sdd_batch {
     int nsm = 1;
     // device: concatenated node arrays and round plan
     int32_t* node_prob = nullptr;
+    int32_t* node_fill = nullptr;    // per node: its problem's fill_task_paths
+    int32_t* node_fill_host = nullptr;
     int32_t* node_role = nullptr;    // concatenated sampling roles (null: every node by Monte Carlo)
     double *shift = nullptr, *acc = nullptr, *est = nullptr, *se = nullptr;
     int64_t *n_done = nullptr, *steps = nullptr, *paths_run = nullptr, *next_total = nullptr;
     int64_t *p_begin = nullptr, *p_count = nullptr, *task_off = nullptr;
-    int32_t *node_of = nullptr, *n_active = nullptr, *task_counter = nullptr;
+    int32_t *node_of = nullptr, *task_len = nullptr, *n_active = nullptr, *task_counter = nullptr;
     TaskSlot* slots = nullptr;
     // device records refreshed every step, and their pinned host sources
     void* mcprob_dev = nullptr;
@@ -158,6 +160,8 @@ void refresh_records(sdd_batch* b)
 {
     for (int i = 0; i < b->n; ++i) {
         const sdd_problem* p = b->probs[i];
+        const int32_t fill = p->fill();
+        for (int m = 0; m < p->M; ++m) b->node_fill_host[b->node_off[i] + m] = fill;
         if (b->fp64) {
             McProblem<double> R = mc_problem<double>(p);
             R.node_offset = b->node_off[i];
@@ -197,6 +201,7 @@ sdd_status launch_batch_mc(sdd_batch* b)
     P.shift = b->shift;
     P.node_of = b->node_of; P.p_begin = b->p_begin; P.p_count = b->p_count; P.task_off = b->task_off;
     P.n_active = b->n_active; P.task_counter = b->task_counter; P.slots = b->slots;
+    P.task_len = b->task_len;
     P.task_paths = b->task_paths;
     B_CK(launch_mc<T>(P, b->acc_mode, false, true, b->mc_grid, b->stream, b->tpb, b->mc_mode));
     return SDD_OK;
@@ -213,13 +218,22 @@ void set_block_size(sdd_batch* b, int tpb, int bps = 0)
     b->mc_grid = b->nsm * (b->bps > 0 ? b->bps : b->max_bps);
 }
 
+// The per-step records and per-node task sizes the round plan and the path kernel read.
+cudaError_t upload_task_sizes(sdd_batch* b)
+{
+    const size_t rec = b->fp64 ? sizeof(McProblem<double>) : sizeof(McProblem<float>);
+    cudaError_t e = cudaMemcpyAsync(b->mcprob_dev, b->mcprob_host, rec * b->n, cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess && b->M > 0)
+        e = cudaMemcpyAsync(b->node_fill, b->node_fill_host, 4 * (size_t)b->M, cudaMemcpyHostToDevice, b->stream);
+    return e;
+}
+
 // The launches of one step.  `capturing`: only fixed-N work (no host round trip).  first_plan:
 // stop after planning the first Monte Carlo round (used to time the path kernel).
 sdd_status record_step(sdd_batch* b, bool first_plan = false)
 {
-    const size_t rec = b->fp64 ? sizeof(McProblem<double>) : sizeof(McProblem<float>);
     int64_t launches = 0;
-    B_CK(cudaMemcpyAsync(b->mcprob_dev, b->mcprob_host, rec * b->n, cudaMemcpyHostToDevice, b->stream));
+    B_CK(upload_task_sizes(b));
     B_CK(cudaMemcpyAsync(b->solve_dev, b->solve_host, sizeof(SolveParams) * b->n, cudaMemcpyHostToDevice,
                          b->stream));
     B_CK(cudaMemcpyAsync(b->t_dev, b->t_host, sizeof(double) * b->n, cudaMemcpyHostToDevice, b->stream));
@@ -244,6 +258,7 @@ sdd_status record_step(sdd_batch* b, bool first_plan = false)
         PP.p_begin = b->p_begin; PP.p_count = b->p_count; PP.task_off = b->task_off;
         PP.n_active = b->n_active; PP.task_counter = b->task_counter;
         PP.task_paths = b->task_paths;
+        PP.node_fill = b->node_fill; PP.task_len = b->task_len;
         ReduceParams RP{};
         RP.node_of = b->node_of; RP.p_count = b->p_count; RP.task_off = b->task_off; RP.n_active = b->n_active;
         RP.slots = b->slots; RP.shift = b->shift; RP.acc = b->acc; RP.n_done = b->n_done; RP.steps = b->steps;
@@ -383,10 +398,10 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
     cudaError_t e = cudaSuccess;
 #define ALLOC(ptr, bytes) if (e == cudaSuccess) e = b->dalloc(&(ptr), (bytes))
 #define HALLOC(ptr, bytes) if (e == cudaSuccess) e = b->halloc(&(ptr), (bytes))
-    ALLOC(b->node_prob, M * 4); ALLOC(b->shift, M * 16); ALLOC(b->acc, M * 32); ALLOC(b->est, M * 16);
+    ALLOC(b->node_prob, M * 4); ALLOC(b->node_fill, M * 4); ALLOC(b->shift, M * 16); ALLOC(b->acc, M * 32); ALLOC(b->est, M * 16);
     ALLOC(b->se, M * 16); ALLOC(b->n_done, M * 8); ALLOC(b->steps, M * 8); ALLOC(b->paths_run, M * 8);
     ALLOC(b->next_total, M * 8); ALLOC(b->p_begin, M * 8); ALLOC(b->p_count, M * 8);
-    ALLOC(b->task_off, (M + 1) * 8); ALLOC(b->node_of, M * 4); ALLOC(b->n_active, 16);
+    ALLOC(b->task_off, (M + 1) * 8); ALLOC(b->node_of, M * 4); ALLOC(b->task_len, M * 4); ALLOC(b->n_active, 16);
     ALLOC(b->task_counter, 16); ALLOC(b->slots, M * kSlotsPerNode * sizeof(TaskSlot));
     ALLOC(b->mcprob_dev, rec * n); ALLOC(b->solve_dev, sizeof(SolveParams) * n); ALLOC(b->t_dev, 8 * n);
     ALLOC(b->sub_off_dev, 4 * (n + 1));
@@ -395,6 +410,7 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
     if (sampled_any) ALLOC(b->node_role, M * 4);
     HALLOC(b->mcprob_host, rec * n); HALLOC(b->solve_host, sizeof(SolveParams) * n); HALLOC(b->t_host, 8 * n);
     HALLOC(b->h_n_active, 32); HALLOC(b->rec_host, sizeof(BatchRec) * n);
+    HALLOC(b->node_fill_host, M * 4);
 #undef ALLOC
 #undef HALLOC
     if (e == cudaSuccess) e = cudaEventCreate(&b->ev0);
@@ -650,7 +666,11 @@ sdd_status sdd_batch_tune_mc(sdd_batch* b, int32_t tune_paths_per_task, sdd_mc_c
             const int T = tune_paths_per_task ? tps[a] : tp0;
             const int64_t round = n0 < (int64_t)kTasksPerRound * T ? n0 : (int64_t)kTasksPerRound * T;
             PP.task_paths = T;
+            PP.node_fill = b->node_fill; PP.task_len = b->task_len;
             b->task_paths = T;  // read by launch_batch_mc; restored or replaced below
+            for (sdd_problem* p : b->probs) p->task_paths = T;
+            refresh_records(b);  // nothing in flight: the previous candidate's event was waited for
+            ce = upload_task_sizes(b);
             for (int k = 0; k < 3 && st == SDD_OK && ce == cudaSuccess; ++k) {
                 set_block_size(b, tpbs[k]);
                 const int max_bps = b->max_bps;

@@ -129,6 +129,45 @@ enum AccMode { kAcc64 = 0, kAccKahan32 = 1 };
 // most kTasksPerRound tasks, so the task slots per node stay the same.
 constexpr int kPathsPerTask = 2048;
 constexpr int kTasksPerRound = 256;
+// Task size of a problem whose tasks of tp paths would leave most of the GPU's warps without one
+// (`nodes` interface nodes, sampled or not, of n0 paths): the largest halving of tp, down to one path per
+// lane, that makes the number of tasks wanted; 0 where tp already does.  A function of the problem
+// alone, so that a node's sums group alike in every launch it shares.
+// Paths that may exit have different lengths, and a short task idles its lanes behind its longest
+// path, so there the count wanted is low: in FP32 2432 tasks, half the resident warps (form 1,
+// 200 x 141 nodes, 1000 paths of about 97 substeps a node: 0.91 ms against 1.41 ms unsplit; four
+// times as many tasks win 4 % more there and cost up to 8 % where paths are shorter), in FP64 608,
+// one per SM sub-partition, whose unit a few warps fill (33 x 33, 61 x 1000 paths: 0.47 ms against
+// 1.54).  FP32 paths of form 0 are the most uneven, exit after a few substeps and gain nothing
+// (sixteen bump problems in a batch: 20.3 ms against 20.6), so they keep tp, as do compensated
+// FP32 sums, whose value depends on the grouping beyond the FP64 rounding.
+// Periodic paths all run K substeps and leave no lane idle: many tasks even out the last wave
+// (2032 x 4000 paths, K = 100: 7.8 ms against 10.2), as long as a task keeps 128 substeps a lane
+// to spread its own start and reduction over.
+inline int fill_task_paths(int64_t nodes, int64_t n0, int tp, bool fp64, int acc_mode, int form, int periodic,
+                           int K)
+{
+    if (!fp64 && (acc_mode == kAccKahan32 || (form == 0 && !periodic))) return 0;
+    int64_t want = fp64 ? 608 : 2432;
+    int t = tp;
+    if (periodic && K > 1) {
+        want = 32768;
+        while (t > 32 && (int64_t)t * K >= 2 * 4096 && nodes * ((n0 + t - 1) / t) < want) t >>= 1;
+    } else {
+        while (t > 32 && nodes * ((n0 + t - 1) / t) < want) t >>= 1;
+    }
+    return t < tp ? t : 0;
+}
+
+// Task size of a chunk of `count` paths: the problem's fill size (0: tp), doubled while the chunk
+// would take more than a round's tasks per node.
+__host__ __device__ __forceinline__ int chunk_task_paths(int64_t count, int fill, int tp)
+{
+    int t = fill > 0 && fill < tp ? fill : tp;
+    while (t < tp && count > (int64_t)kTasksPerRound * t) t <<= 1;
+    return t;
+}
+
 constexpr int kRoundsAhead = 2;  // adaptive Monte Carlo rounds queued ahead of the host's decision
 // Adaptive chunk totals are multiples of this many paths.
 constexpr int64_t kAdaptiveGranule = 1024;
@@ -173,7 +212,8 @@ template <typename T> struct McParams {
     const int32_t* n_active;   // device scalar
     int32_t* task_counter;     // dynamic task dispenser (reset by the plan kernel)
     TaskSlot* slots;           // one per task
-    int32_t task_paths;        // paths per task (0: kPathsPerTask)
+    const int32_t* task_len;   // paths per task of each active node (plan kernel), or null:
+    int32_t task_paths;        //   of every node
     // debug records (null unless the debug variant runs; single-problem launches only)
     double* dbg_val;
     int32_t* dbg_steps;
@@ -200,6 +240,9 @@ struct PlanParams {
     int64_t max_tasks;         // > 0: cap on the round's tasks (nodes in planning order)
     int32_t task_paths;        // paths per task (0: kPathsPerTask); a node takes at most
                                // kTasksPerRound tasks per round
+    int32_t fill;              // single problems: fill_task_paths of the problem (0: task_paths)
+    const int32_t* node_fill;  // several problems: the same per node (null: fill)
+    int32_t* task_len;         // out (nullable): paths per task of each active node
 };
 
 struct ReduceParams {

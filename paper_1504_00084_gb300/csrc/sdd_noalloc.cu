@@ -184,7 +184,7 @@ bool on_device(const void* p)
 }
 
 template <typename T>
-sdd_status run(const sdd_params* P, const Buffers& b, int M, int acc_mode, int32_t step_index,
+sdd_status run(const sdd_params* P, const Buffers& b, int M, int acc_mode, int task_paths, int32_t step_index,
                cudaStream_t s)
 {
     int dev = 0, nsm = 1;
@@ -212,11 +212,13 @@ sdd_status run(const sdd_params* P, const Buffers& b, int M, int acc_mode, int32
     mp.shift = b.shift;
     mp.node_of = b.node_of; mp.p_begin = b.p_begin; mp.p_count = b.p_count; mp.task_off = b.task_off;
     mp.n_active = b.n_active; mp.task_counter = b.task_counter; mp.slots = b.slots;
+    mp.task_paths = task_paths;
 
     PlanParams pp{};
     pp.M = M; pp.n_done = b.n_done; pp.next_total = b.next_total; pp.node_of = b.node_of;
     pp.p_begin = b.p_begin; pp.p_count = b.p_count; pp.task_off = b.task_off;
     pp.n_active = b.n_active; pp.task_counter = b.task_counter;
+    pp.task_paths = task_paths;
     ReduceParams rp{};
     rp.node_of = b.node_of; rp.p_count = b.p_count; rp.task_off = b.task_off; rp.n_active = b.n_active;
     rp.slots = b.slots; rp.shift = b.shift; rp.acc = b.acc; rp.n_done = b.n_done; rp.steps = b.steps;
@@ -262,12 +264,20 @@ extern "C" sdd_status sdd_interface_mc_noalloc(const sdd_params* P, const double
     if (M < 0 || M > (int64_t(1) << 20) || N > (int64_t(1) << 24)) return SDD_ERR_INVALID_ARG;
     if (M > 0 && (!est_xy || !se_xy)) return SDD_ERR_INVALID_ARG;
     const int64_t chunk = P->paths_per_node < kMaxChunk ? P->paths_per_node : kMaxChunk;
-    const int64_t slots = M * ((chunk + kPathsPerTask - 1) / kPathsPerTask);
     const bool fp64 = P->precision == SDD_FP64;
+    const int acc_mode = P->precision == SDD_FP32_KAHAN ? kAccKahan32 : kAcc64;
     Buffers b{};
-    Carve sizing{nullptr};
-    if (carve(sizing, b, (size_t)N, (size_t)M, (size_t)slots, fp64 ? 8 : 4, mon_bytes(P->nx, P->ny, fp64)) > kScratchBytes)
-        return SDD_ERR_INVALID_ARG;  // larger than the fixed scratch array
+    // tasks of the size sdd_interface_mc uses, or of twice that and so on until their slots fit
+    int task_paths = chunk_task_paths(chunk, fill_task_paths(M, P->paths_per_node, kPathsPerTask, fp64, acc_mode, P->form,
+                                                             P->periodic, P->substeps), kPathsPerTask);
+    int64_t slots = 0;
+    for (;; task_paths <<= 1) {
+        slots = M * ((chunk + task_paths - 1) / task_paths);
+        Carve sizing{nullptr};
+        if (carve(sizing, b, (size_t)N, (size_t)M, (size_t)slots, fp64 ? 8 : 4, mon_bytes(P->nx, P->ny, fp64)) <= kScratchBytes)
+            break;
+        if (task_paths >= kPathsPerTask) return SDD_ERR_INVALID_ARG;  // larger than the fixed scratch array
+    }
     if (!on_device(x) || !on_device(y) || !on_device(omega)) return SDD_ERR_INVALID_ARG;
     if (M == 0) return SDD_OK;  // one Dirichlet subdomain: no interface node, nothing to write
     if (!on_device(est_xy) || !on_device(se_xy)) return SDD_ERR_INVALID_ARG;
@@ -288,9 +298,8 @@ extern "C" sdd_status sdd_interface_mc_noalloc(const sdd_params* P, const double
     pr.om64 = b.om64; pr.wxi64 = b.wxi64; pr.weta64 = b.weta64; pr.mon = b.mon; pr.disp = b.disp;
     if (launch_prep(pr, s) != cudaSuccess) return SDD_ERR_CUDA;
     if (launch_shift(b.nodes, (int)M, P->nx, x, y, b.shift, s) != cudaSuccess) return SDD_ERR_CUDA;
-    const int acc_mode = P->precision == SDD_FP32_KAHAN ? kAccKahan32 : kAcc64;
-    const sdd_status r = fp64 ? run<double>(P, b, (int)M, acc_mode, step_index, s)
-                              : run<float>(P, b, (int)M, acc_mode, step_index, s);
+    const sdd_status r = fp64 ? run<double>(P, b, (int)M, acc_mode, task_paths, step_index, s)
+                              : run<float>(P, b, (int)M, acc_mode, task_paths, step_index, s);
     if (r != SDD_OK) return r;
     if (launch_output((int)M, b.acc, b.n_done, b.shift, est_xy, se_xy, s) != cudaSuccess) return SDD_ERR_CUDA;
     return SDD_OK;

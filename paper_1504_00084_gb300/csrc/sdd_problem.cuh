@@ -29,6 +29,12 @@ struct sdd_problem {
     int mc_blocks_per_sm = 1;       // resident path-kernel blocks per SM (sdd_set_mc_config)
     int mc_max_blocks_per_sm = 1;   // the register limit of the path kernel
     int task_paths = sdd::kPathsPerTask;  // paths per warp task (sdd_set_mc_config)
+    // the task size that fills the GPU at this problem's size (fill_task_paths)
+    int fill() const
+    {
+        return sdd::fill_task_paths(M, prm.paths_per_node, task_paths, fp64, acc_mode,
+                                    prm.form, prm.periodic, prm.substeps);
+    }
     int nsm = 1;
     bool fp64 = true;
     int acc_mode = sdd::kAcc64;
@@ -57,6 +63,7 @@ struct sdd_problem {
     int64_t *n_done = nullptr, *steps = nullptr, *paths_run = nullptr, *next_total = nullptr;
     int32_t* node_of = nullptr;
     int64_t *p_begin = nullptr, *p_count = nullptr, *task_off = nullptr;
+    int32_t *task_len = nullptr;
     int32_t *n_active = nullptr, *task_counter = nullptr;
     sdd::TaskSlot* slots = nullptr;
     int64_t slot_cap = 0;

@@ -103,10 +103,11 @@ struct sdd_server {
     int mc_grid = 1;
     // node pool (device)
     int32_t* node_prob = nullptr;
+    int32_t* node_fill = nullptr;    // per node: its request's fill_task_paths
     double *shift = nullptr, *acc = nullptr, *est = nullptr, *se = nullptr;
     int64_t *n_done = nullptr, *steps = nullptr, *paths_run = nullptr, *next_total = nullptr;
     int64_t *p_begin = nullptr, *p_count = nullptr, *task_off = nullptr;
-    int32_t *node_of = nullptr, *n_active = nullptr, *task_counter = nullptr;
+    int32_t *node_of = nullptr, *task_len = nullptr, *n_active = nullptr, *task_counter = nullptr;
     TaskSlot* slots = nullptr;
     int2* slot_range = nullptr;
     int32_t* pending = nullptr;
@@ -352,13 +353,14 @@ sdd_status admit(sdd_server* s, Request* r)
         const int64_t o = r->off;
         S_CK(launch_shift(p->nodes, r->M, r->prm.nx, p->x, p->y, s->shift + 2 * o, s->stream));
         fill_i32_kernel<<<(r->M + 255) / 256, 256, 0, s->stream>>>(s->node_prob + o, r->M, r->slot);
+        fill_i32_kernel<<<(r->M + 255) / 256, 256, 0, s->stream>>>(s->node_fill + o, r->M, p->fill());
         S_CK(cudaGetLastError());
         const bool adaptive = s->prm.se_target > 0;
         const int64_t n0 = s->prm.paths_per_node;
         const int64_t maxp = adaptive ? s->prm.max_paths_per_node : n0;
         S_CK(launch_mc_init(r->M, n0, maxp, s->acc + 4 * o, s->n_done + o, s->steps + o, s->paths_run + o,
                             s->next_total + o, s->stream, p->n_interp > 0 ? p->iface_role : nullptr));
-        s->st.kernel_launches += 3;
+        s->st.kernel_launches += 4;
     }
     if (s->fp64) write_record<double>(s, r); else write_record<float>(s, r);
     const size_t rec = s->fp64 ? sizeof(McProblem<double>) : sizeof(McProblem<float>);
@@ -414,6 +416,7 @@ sdd_status launch_round(sdd_server* s, int hw)
     P.shift = s->shift;
     P.node_of = s->node_of; P.p_begin = s->p_begin; P.p_count = s->p_count; P.task_off = s->task_off;
     P.n_active = s->n_active; P.task_counter = s->task_counter; P.slots = s->slots;
+    P.task_len = s->task_len; P.task_paths = kPathsPerTask;
     // the problem switches, when every running request shares them (the path kernel then has
     // them compiled in; each request's results are the same either way)
     int mode = -1;
@@ -497,10 +500,10 @@ sdd_status sdd_server_create(const sdd_server_params* params, void* stream, sdd_
     cudaError_t e = cudaSuccess;
 #define ALLOC(ptr, bytes) if (e == cudaSuccess) e = s->dalloc(&(ptr), (bytes))
 #define HALLOC(ptr, bytes) if (e == cudaSuccess) e = s->halloc(&(ptr), (bytes))
-    ALLOC(s->node_prob, M * 4); ALLOC(s->shift, M * 16); ALLOC(s->acc, M * 32); ALLOC(s->est, M * 16);
+    ALLOC(s->node_prob, M * 4); ALLOC(s->node_fill, M * 4); ALLOC(s->shift, M * 16); ALLOC(s->acc, M * 32); ALLOC(s->est, M * 16);
     ALLOC(s->se, M * 16); ALLOC(s->n_done, M * 8); ALLOC(s->steps, M * 8); ALLOC(s->paths_run, M * 8);
     ALLOC(s->next_total, M * 8); ALLOC(s->p_begin, M * 8); ALLOC(s->p_count, M * 8);
-    ALLOC(s->task_off, (M + 1) * 8); ALLOC(s->node_of, M * 4); ALLOC(s->n_active, 16);
+    ALLOC(s->task_off, (M + 1) * 8); ALLOC(s->node_of, M * 4); ALLOC(s->task_len, M * 4); ALLOC(s->n_active, 16);
     ALLOC(s->task_counter, 16); ALLOC(s->slots, M * kSlotsPerNode * sizeof(TaskSlot));
     ALLOC(s->slot_range, R * sizeof(int2)); ALLOC(s->pending, (R + 1) * 4); ALLOC(s->records, rec * R);
     ALLOC(s->range_off, (R + 1) * 4); ALLOC(s->range_pre, (R + 1) * 4); ALLOC(s->slot_bad, R * 4);
@@ -647,6 +650,7 @@ sdd_status sdd_server_progress(sdd_server* s, int32_t* n_running, int32_t* n_que
             PP.p_begin = s->p_begin; PP.p_count = s->p_count; PP.task_off = s->task_off;
             PP.n_active = s->n_active; PP.task_counter = s->task_counter;
             PP.range_off = s->range_off; PP.range_pre = s->range_pre; PP.n_ranges = nr;
+            PP.node_fill = s->node_fill; PP.task_len = s->task_len;
             PP.max_tasks = (s->prm.round_paths + kPathsPerTask - 1) / kPathsPerTask;
             S_CK(launch_plan(PP, s->stream));
             slot_pending_kernel<<<(R * 32 + 255) / 256, 256, 0, s->stream>>>(s->slot_range, R, s->n_done,
