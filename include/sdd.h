@@ -56,7 +56,8 @@ typedef enum {
 enum { SDD_FORM_DIV = 0, SDD_FORM_WINSLOW = 1 };
 
 /* Working precision of the paths and of the estimator sums (subdomain solves: FP64 PCG for
- * SDD_FP64, FP32 PCG with FP64 residuals and iterative refinement otherwise). */
+ * SDD_FP64, its multigrid preconditioner in FP32 for subdomains up to about 128 x 128; FP32 PCG with
+ * FP64 residuals and iterative refinement otherwise). */
 enum { SDD_FP64 = 0, SDD_FP32_ACC64 = 1, SDD_FP32_KAHAN = 2 };
 
 /* Monitor (mesh density) kinds, evaluated on the current physical mesh (x, y) at t^n. */

@@ -425,12 +425,9 @@ sdd_status run_solve(sdd_problem* p)
     if (!p->solve_ev[0]) SDD_CK(cudaEventCreate(&p->solve_ev[0]));
     if (!p->solve_ev[1]) SDD_CK(cudaEventCreate(&p->solve_ev[1]));
     SDD_CK(cudaEventRecord(p->solve_ev[0], p->stream));
-    if (!p->h_items.empty())
-        SDD_CK(launch_solve_items(S, p->solve_items, (int)p->h_items.size(), p->fp64, p->stream));
-    else
-        SDD_CK(launch_solve(S, p->fp64, p->stream));
+    SDD_CK(launch_solve(S, p->plan, p->chip_items, p->solve_items, p->fp64, p->stream));
     SDD_CK(cudaEventRecord(p->solve_ev[1], p->stream));
-    p->launches += 2;
+    p->launches += 1 + (p->prm.subdomain_scheme == 1 ? 1 : (int)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1));
     const int ns = p->prm.px * p->prm.py;
     std::vector<int32_t> it(ns), ou(ns), ok(ns);
     std::vector<double> rs(ns);
@@ -512,7 +509,8 @@ void problem_arrays(sdd_problem* p, bool with_mc, F&& f)
     f((void**)&p->quality, (N + 2) * 8);
     f((void**)&p->mg, p->mg_stride * ns);
     f((void**)&p->bad, 16);
-    f((void**)&p->solve_items, (p->h_items.size() + 1) * sizeof(SolveItem));
+    f((void**)&p->solve_items, (p->plan.items.size() + 1) * sizeof(SolveItem));
+    f((void**)&p->chip_items, (p->plan.chip_items.size() + 1) * sizeof(int2));
     const size_t nb = 2 * (size_t)q.nx + 2 * (size_t)q.ny;
     f((void**)&p->bnd64, nb * 8);
     f((void**)&p->bnd, nb * rs);
@@ -543,17 +541,11 @@ sdd_problem* problem_shell(const sdd_params& prm, cudaStream_t stream)
             if (m > mg) mg = m;
         }
     p->mg_stride = mg;
-    // subdomains by interior size, largest first; large ones are solved by a cluster of CTAs
-    std::vector<std::pair<int64_t, int2>> subs;
-    for (int k = 0; k < prm.px * prm.py; ++k) {
-        const int I = k % prm.px, J = k / prm.px;
-        const int64_t wi = split_line(I + 1, prm.nx, prm.px) - split_line(I, prm.nx, prm.px) - 1;
-        const int64_t wj = split_line(J + 1, prm.ny, prm.py) - split_line(J, prm.ny, prm.py) - 1;
-        subs.push_back({wi * wj, make_int2(0, k)});
+    if (prm.subdomain_scheme == 0) {
+        std::vector<SolveSub> subs;
+        solve_subs(0, prm.nx, prm.ny, prm.px, prm.py, subs);
+        p->plan = solve_plan(subs, p->fp64);
     }
-    std::stable_sort(subs.begin(), subs.end(), [](const std::pair<int64_t, int2>& a,
-                                                  const std::pair<int64_t, int2>& c) { return a.first > c.first; });
-    if (prm.subdomain_scheme == 0) p->h_items = solve_items(subs);
     p->stats.M = p->M;
     p->stats.t = prm.t0;
     return p;
@@ -607,8 +599,11 @@ sdd_status sdd_alloc_problem(const sdd_params& prm, cudaStream_t stream, bool wi
     if (e == cudaSuccess && p->n_interp > 0)
         e = cudaMemcpyAsync(p->interp, p->h_interp.data(), (size_t)p->n_interp * sizeof(InterpRule),
                             cudaMemcpyHostToDevice, p->stream);
-    if (e == cudaSuccess && !p->h_items.empty())
-        e = cudaMemcpyAsync(p->solve_items, p->h_items.data(), p->h_items.size() * sizeof(SolveItem),
+    if (e == cudaSuccess && !p->plan.items.empty())
+        e = cudaMemcpyAsync(p->solve_items, p->plan.items.data(), p->plan.items.size() * sizeof(SolveItem),
+                            cudaMemcpyHostToDevice, p->stream);
+    if (e == cudaSuccess && !p->plan.chip_items.empty())
+        e = cudaMemcpyAsync(p->chip_items, p->plan.chip_items.data(), p->plan.chip_items.size() * sizeof(int2),
                             cudaMemcpyHostToDevice, p->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);  // p->ij is pageable host memory
     if (e != cudaSuccess) {

@@ -70,8 +70,9 @@ struct sdd_batch {
     double* t_host = nullptr;
     int32_t* sub_off_dev = nullptr;
     int2* order_dev = nullptr;       // solve CTAs: (problem, subdomain), largest subdomains first
-    SolveItem* items_dev = nullptr;  // cooperative solve items (n_items > 0: large subdomains present)
-    int n_items = 0;
+    SolvePlan plan;                  // how the backward-Euler subdomains are solved
+    SolveItem* items_dev = nullptr;
+    int2* chip_items_dev = nullptr;
     // batched per-problem launches: records (refreshed every step) and per-problem block offsets
     BatchRec* rec_dev = nullptr;
     BatchRec* rec_host = nullptr;
@@ -320,23 +321,13 @@ sdd_status record_step(sdd_batch* b, bool first_plan = false)
     launches += 1 + (b->M > 0 ? 1 : 0);
     B_CK(launch_faces_batch(b->solve_dev, b->blk_off_dev, b->n, b->total_blocks, fp64_inner, b->stream));
     launches += 1;
-    bool any_be = false, any_fe = false;
-    for (const sdd_problem* p : b->probs) {
-        any_be = any_be || p->prm.subdomain_scheme == 0;
-        any_fe = any_fe || p->prm.subdomain_scheme == 1;
-    }
+    bool any_fe = false;
+    for (const sdd_problem* p : b->probs) any_fe = any_fe || p->prm.subdomain_scheme == 1;
     B_CK(cudaEventRecord(b->sev0, b->stream));
-    if (b->n_items > 0) {
-        B_CK(launch_solve_batch_items(b->solve_dev, b->items_dev, b->n_items, fp64_inner, b->stream));
-        if (any_fe)
-            B_CK(launch_solve_batch(b->solve_dev, b->sub_off_dev, b->n, b->total_subs, fp64_inner, b->stream,
-                                    false, true, b->order_dev));
-    } else {
-        B_CK(launch_solve_batch(b->solve_dev, b->sub_off_dev, b->n, b->total_subs, fp64_inner, b->stream, any_be,
-                                any_fe, b->order_dev));
-    }
+    B_CK(launch_solve_batch(b->solve_dev, b->plan, b->chip_items_dev, b->items_dev, fp64_inner, any_fe, b->order_dev,
+                            b->total_subs, b->stream));
     B_CK(cudaEventRecord(b->sev1, b->stream));
-    launches += (any_be ? 1 : 0) + (any_fe ? 1 : 0);
+    launches += (int64_t)b->plan.chip.size() + (b->plan.items.empty() ? 0 : 1) + (any_fe ? 1 : 0);
     B_CK(launch_copy_back_batch(b->rec_dev, b->blk_off_dev, b->n, b->total_blocks, b->stream));
     launches += 1;
     b->launches_per_step = launches;
@@ -456,15 +447,23 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
         for (const auto& v : subs) order.push_back(v.second);
         e = cudaMemcpy(b->order_dev, order.data(), sizeof(int2) * order.size(), cudaMemcpyHostToDevice);
         // backward-Euler subdomains only: forward-Euler problems run in their own kernel
-        std::vector<std::pair<int64_t, int2>> be;
-        for (const auto& v : subs)
-            if (problems[v.second.x]->prm.subdomain_scheme == 0) be.push_back(v);
-        const std::vector<SolveItem> items = solve_items(be);
-        if (e == cudaSuccess && !items.empty()) {
-            e = b->dalloc(&b->items_dev, sizeof(SolveItem) * items.size());
+        std::vector<SolveSub> be;
+        for (int i = 0; i < n; ++i) {
+            const sdd_params& q = problems[i]->prm;
+            if (q.subdomain_scheme == 0) solve_subs(i, q.nx, q.ny, q.px, q.py, be);
+        }
+        b->plan = solve_plan(be, b->fp64);
+        if (e == cudaSuccess && !b->plan.items.empty()) {
+            e = b->dalloc(&b->items_dev, sizeof(SolveItem) * b->plan.items.size());
             if (e == cudaSuccess)
-                e = cudaMemcpy(b->items_dev, items.data(), sizeof(SolveItem) * items.size(), cudaMemcpyHostToDevice);
-            b->n_items = (int)items.size();
+                e = cudaMemcpy(b->items_dev, b->plan.items.data(), sizeof(SolveItem) * b->plan.items.size(),
+                               cudaMemcpyHostToDevice);
+        }
+        if (e == cudaSuccess && !b->plan.chip_items.empty()) {
+            e = b->dalloc(&b->chip_items_dev, sizeof(int2) * b->plan.chip_items.size());
+            if (e == cudaSuccess)
+                e = cudaMemcpy(b->chip_items_dev, b->plan.chip_items.data(), sizeof(int2) * b->plan.chip_items.size(),
+                               cudaMemcpyHostToDevice);
         }
     }
     if (e == cudaSuccess && sampled_any && b->M > 0)

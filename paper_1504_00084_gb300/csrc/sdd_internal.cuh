@@ -7,8 +7,8 @@
 //                 Euler-Maruyama, exit tests, terminal values, deterministic reductions,
 //                 round plan, interface-sampling interpolation
 //   sdd_solve.cu  subdomain solves (Sec. 3.5): backward Euler by multigrid-preconditioned CG with
-//                 FP64 refinement, or forward-Euler substeps; one CTA (or a cluster of four,
-//                 for large subdomains) per subdomain
+//                 FP64 refinement, on chip where a subdomain fits (sdd_chip.cuh) or from global
+//                 memory, or forward-Euler substeps; one CTA or a cluster per subdomain
 // Host code:
 //   sdd_api.cu    the C ABI of single problems; sdd_batch.cu batches; sdd_server.cu serving;
 //                 sdd_noalloc.cu the allocation-free interface Monte Carlo
@@ -336,10 +336,27 @@ struct SolveItem {
     int32_t prob, sub, width, pad;
 };
 
-// Work items of a solve launch over the given subdomains (problem, subdomain, interior unknowns),
-// in the given order: a cooperative subdomain takes a whole cluster; the others are packed
-// kCoopWidth to a cluster.  Empty when no subdomain is cooperative (the one-CTA kernels serve).
-std::vector<SolveItem> solve_items(const std::vector<std::pair<int64_t, int2>>& subs);
+// A subdomain to be solved by backward Euler: subdomain `sub` of problem `prob`, ni x nj interior nodes.
+struct SolveSub {
+    int32_t prob, sub, ni, nj;
+};
+// One launch of the on-chip solve kernel (sdd_chip.cuh): `count` subdomains from items[first] on, each
+// by cw CTAs of nw warps, `slots` nodes a thread, with smem bytes of dynamic shared memory.
+struct ChipLaunch {
+    int cw, nw, slots, smem, first, count;
+};
+// How a list of subdomains is solved: those that fit on chip by class of team, the others from global
+// memory (SolveItem: a cooperative subdomain takes a whole cluster, the others are packed kCoopWidth
+// to a cluster).
+struct SolvePlan {
+    std::vector<ChipLaunch> chip;
+    std::vector<int2> chip_items;   // (problem, subdomain)
+    std::vector<SolveItem> items;
+};
+// The plan of the subdomains of one problem's split (solve_subs), or of several problems'.
+SolvePlan solve_plan(std::vector<SolveSub> subs, bool fp64);
+// Subdomains of an nx x ny grid split px x py, appended to `subs` as problem `prob`.
+void solve_subs(int prob, int nx, int ny, int px, int py, std::vector<SolveSub>& subs);
 
 // Multigrid hierarchy of an n x m subdomain interior: the coarse grid keeps the nodes of odd
 // index, (n - 1) / 2 of them for odd n and n / 2 for even n (then the last coarse node lies one
@@ -404,7 +421,9 @@ template <typename T> int mc_max_blocks_per_sm(int acc_mode, bool debug, bool ba
 cudaError_t launch_reduce(const ReduceParams& P, int M, cudaStream_t s);
 cudaError_t launch_output(int M, const double* acc, const int64_t* n_done, const double* shift,
                           double* est, double* se, cudaStream_t s);
-cudaError_t launch_solve(const SolveParams& P, bool fp64_inner, cudaStream_t s);
+// Face coefficients and subdomain solves of one problem (plan's items in device memory).
+cudaError_t launch_solve(const SolveParams& P, const SolvePlan& plan, const int2* chip_items, const SolveItem* items,
+                         bool fp64_inner, cudaStream_t s);
 cudaError_t launch_faces(const SolveParams& P, bool fp64_inner, cudaStream_t s);
 // Batched launches of a batch step (blk_off: per-problem block offsets of grid-sized work, n + 1
 // entries, blocks of 256 threads as batch_blocks gives them; node work over the concatenated nodes).
@@ -417,20 +436,14 @@ cudaError_t launch_scatter_batch(const BatchRec* R, const int32_t* blk_off, int 
 cudaError_t launch_copy_back_batch(const BatchRec* R, const int32_t* blk_off, int n, int total_blocks, cudaStream_t s);
 cudaError_t launch_faces_batch(const SolveParams* probs, const int32_t* blk_off, int n, int total_blocks,
                                bool fp64_inner, cudaStream_t s);
-// order (nullable): (problem, subdomain) of each CTA
-cudaError_t launch_solve_batch(const SolveParams* probs, const int32_t* sub_off, int n, int total_subs,
-                               bool fp64_inner, cudaStream_t s, bool any_be = true, bool any_fe = false,
-                               const int2* order = nullptr);
+// Backward-Euler solves of a batch (plan's items in device memory), then its forward-Euler problems
+// (any_fe; order: (problem, subdomain) of each CTA).
+cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const int2* chip_items,
+                               const SolveItem* items, bool fp64_inner, bool any_fe, const int2* order, int total_subs,
+                               cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, const uint32_t* key, int64_t n, uint32_t* out,
                           cudaStream_t s);
 cudaError_t launch_unit_math(const uint32_t* w, int64_t n, float* out, cudaStream_t s);
-// Cooperative solve launches (items from solve_items); the single-problem one also computes the
-// face coefficients first, as launch_solve does.
-cudaError_t launch_solve_items(const SolveParams& P, const SolveItem* items, int n_items, bool fp64_inner,
-                               cudaStream_t s);
-cudaError_t launch_solve_batch_items(const SolveParams* probs, const SolveItem* items, int n_items,
-                                     bool fp64_inner, cudaStream_t s);
-
 // Host/device shared scheduling rule of the adaptive estimator.
 __host__ __device__ inline int64_t adaptive_next_total(int64_t n_done, double se, double target,
                                                        int64_t max_paths)

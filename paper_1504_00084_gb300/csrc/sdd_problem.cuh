@@ -73,8 +73,9 @@ struct sdd_problem {
     void *ce = nullptr, *cn = nullptr, *vec = nullptr;
     void* mg = nullptr;             // multigrid workspace, mg_stride bytes per subdomain
     size_t mg_stride = 0;
-    std::vector<sdd::SolveItem> h_items;  // cooperative solve items (empty: one CTA per subdomain)
+    sdd::SolvePlan plan;            // how the subdomains are solved (backward Euler)
     sdd::SolveItem* solve_items = nullptr;
+    int2* chip_items = nullptr;
     int32_t *st_iters = nullptr, *st_outer = nullptr, *st_ok = nullptr;
     double* st_res = nullptr;
     double* quality = nullptr;      // (nx-1)(ny-1) cell qualities + 2 stats

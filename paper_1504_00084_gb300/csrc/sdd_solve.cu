@@ -7,8 +7,9 @@
 //   d_P = 1 (tau x_t = div(omega grad x))  or  omega_P (the paper's Eq. 4 form),
 // a symmetric positive-definite system, for both mesh components at once.
 //
-// One CTA of 512 threads per subdomain, two per SM, or a cluster of CTAs for a large subdomain
-// (solve_item).  Outer loop in FP64: residual b - A x of the current iterate (rims
+// Subdomains that fit on chip (up to about 64 x 64 unknowns in one CTA and 256 x 256 in a cluster)
+// are solved in shared memory and registers by sdd_chip.cuh.  The rest work from global memory, one
+// CTA of 512 threads per subdomain, two per SM, or a cluster of CTAs for a large one (solve_item).  Outer loop in FP64: residual b - A x of the current iterate (rims
 // included), stop when ||r||_2 <= rtol ||b||_2 for both components.  Inner solve A e = r by
 // conjugate gradients in the inner precision (FP32 for the FP32 modes, FP64 otherwise),
 // preconditioned by one symmetric multigrid V-cycle, then x += e (iterative refinement).
@@ -25,6 +26,10 @@
 // block trees: the solve is deterministic.
 #include <cooperative_groups.h>
 #include <math.h>
+
+#include <algorithm>
+#include <mutex>
+#include <set>
 
 #include "sdd_internal.cuh"
 
@@ -746,65 +751,22 @@ __device__ __forceinline__ void solve_body(const Team<CW>& tm, const SolveParams
 template <typename TI, int CW>
 __device__ SDD_SOLVE_SUB_ATTR void solve_sub(const Team<CW> tm, const SolveParams& P, int sub, double* sh);
 
-template <typename TI>
-__global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) solve_kernel(const __grid_constant__ SolveParams P)
-{
-    __shared__ double sh[32 * 8 + 8];
-    solve_sub<TI, 1>(Team<1>{0}, P, blockIdx.x, sh);
-}
-
 __global__ void __launch_bounds__(kSolveThreads) fe_kernel(const __grid_constant__ SolveParams P)
 {
     __shared__ double sh[40];
     fe_body(P, blockIdx.x, sh);
 }
 
-// Batched problem record of CTA b: order[b] = (problem, subdomain) when given (largest
-// subdomains first, so the longest CTAs start in the first wave), else problem p with
-// sub_off[p] <= b < sub_off[p + 1].
-__device__ __forceinline__ void batch_lookup(const SolveParams* probs, const int32_t* sub_off, const int2* order,
-                                             int n, SolveParams& sp, int& sub)
-{
-    if (order) {
-        const int2 o = order[blockIdx.x];
-        sp = probs[o.x];
-        sub = o.y;
-        return;
-    }
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (sub_off[mid] <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
-    }
-    sp = probs[lo];
-    sub = (int)blockIdx.x - sub_off[lo];
-}
-
-// Batched forward-Euler subdomains (CTAs of backward-Euler problems return at once).
-__global__ void __launch_bounds__(kSolveThreads) fe_batch_kernel(const SolveParams* probs, const int32_t* sub_off,
-                                                                 const int2* order, int n)
+// Batched forward-Euler subdomains, order[b] = (problem, subdomain) of CTA b (CTAs of backward-Euler
+// problems return at once).
+__global__ void __launch_bounds__(kSolveThreads) fe_batch_kernel(const SolveParams* probs, const int2* order)
 {
     __shared__ double sh[40];
     __shared__ SolveParams sp;
-    __shared__ int sub;
-    if (threadIdx.x == 0) batch_lookup(probs, sub_off, order, n, sp, sub);
+    const int2 o = order[blockIdx.x];
+    if (threadIdx.x == 0) sp = probs[o.x];
     __syncthreads();
-    if (sp.scheme == 1) fe_body(sp, sub, sh);
-}
-
-// Batched: CTA b solves the subdomain batch_lookup assigns it (launches without large subdomains;
-// with them, solve_batch_items_kernel below).
-template <typename TI>
-__global__ void __launch_bounds__(kSolveThreads, kSolveMinBlocks) solve_batch_kernel(const SolveParams* probs,
-                                                                       const int32_t* sub_off, const int2* order,
-                                                                       int n)
-{
-    __shared__ double sh[32 * 8 + 8];
-    __shared__ SolveParams sp;
-    __shared__ int sub;
-    if (threadIdx.x == 0) batch_lookup(probs, sub_off, order, n, sp, sub);
-    __syncthreads();
-    if (sp.scheme == 0) solve_sub<TI, 1>(Team<1>{0}, sp, sub, sh);  // forward-Euler problems: fe_batch_kernel
+    if (sp.scheme == 1) fe_body(sp, o.y, sh);
 }
 
 // The solve of one subdomain, called by every solve kernel.  Inlined into each kernel (measured
@@ -859,54 +821,134 @@ __global__ void __cluster_dims__(kCoopWidth, 1, 1) __launch_bounds__(kSolveThrea
 
 }  // namespace
 
-std::vector<SolveItem> solve_items(const std::vector<std::pair<int64_t, int2>>& subs)
+#include "sdd_chip.cuh"
+
+void solve_subs(int prob, int nx, int ny, int px, int py, std::vector<SolveSub>& subs)
 {
-    std::vector<SolveItem> items;
-    bool any = false;
-    for (const auto& v : subs) any = any || v.first >= kCoopUnknowns;
-    if (!any) return items;
+    for (int k = 0; k < px * py; ++k) {
+        const int I = k % px, J = k / px;
+        subs.push_back(SolveSub{prob, k, split_line(I + 1, nx, px) - split_line(I, nx, px) - 1,
+                                split_line(J + 1, ny, py) - split_line(J, ny, py) - 1});
+    }
+}
+
+SolvePlan solve_plan(std::vector<SolveSub> subs, bool fp64)
+{
+    // longest first; ties in the given order
+    std::stable_sort(subs.begin(), subs.end(), [](const SolveSub& a, const SolveSub& c) {
+        return (int64_t)a.ni * a.nj > (int64_t)c.ni * c.nj;
+    });
+    SolvePlan plan;
+    std::vector<std::pair<ChipLaunch, std::vector<int2>>> classes;
     std::vector<SolveItem> pend;  // subdomains of one CTA each, waiting to fill a cluster
-    for (const auto& v : subs) {
-        if (v.first >= kCoopUnknowns) {
-            for (int r = 0; r < kCoopWidth; ++r) items.push_back(SolveItem{v.second.x, v.second.y, kCoopWidth, 0});
+    for (const SolveSub& v : subs) {
+        ChipLaunch c{};
+        chip_team(v.ni, v.nj, fp64, &c);
+        if (c.cw > 0) {
+            size_t k = 0;
+            while (k < classes.size() && (classes[k].first.cw != c.cw || classes[k].first.nw != c.nw ||
+                                          classes[k].first.slots != c.slots)) ++k;
+            if (k == classes.size()) classes.push_back({c, {}});
+            classes[k].first.smem = std::max(classes[k].first.smem, c.smem);
+            classes[k].second.push_back(make_int2(v.prob, v.sub));
+        } else if ((int64_t)v.ni * v.nj >= kCoopUnknowns) {
+            for (int r = 0; r < kCoopWidth; ++r) plan.items.push_back(SolveItem{v.prob, v.sub, kCoopWidth, 0});
         } else {
-            pend.push_back(SolveItem{v.second.x, v.second.y, 1, 0});
+            pend.push_back(SolveItem{v.prob, v.sub, 1, 0});
             if ((int)pend.size() == kCoopWidth) {
-                items.insert(items.end(), pend.begin(), pend.end());
+                plan.items.insert(plan.items.end(), pend.begin(), pend.end());
                 pend.clear();
             }
         }
     }
     if (!pend.empty()) {
         while ((int)pend.size() < kCoopWidth) pend.push_back(SolveItem{0, 0, 0, 0});
-        items.insert(items.end(), pend.begin(), pend.end());
+        plan.items.insert(plan.items.end(), pend.begin(), pend.end());
     }
-    return items;
+    for (auto& c : classes) {
+        c.first.first = (int)plan.chip_items.size();
+        c.first.count = (int)c.second.size();
+        plan.chip.push_back(c.first);
+        plan.chip_items.insert(plan.chip_items.end(), c.second.begin(), c.second.end());
+    }
+    return plan;
 }
 
-cudaError_t launch_solve_items(const SolveParams& P, const SolveItem* items, int n_items, bool fp64_inner,
-                               cudaStream_t s)
+namespace {
+
+// Raises the kernel's dynamic shared memory limit (and, for wide clusters, allows sizes beyond the
+// portable eight), once per kernel and device.
+cudaError_t chip_allow(const void* fn, bool cluster)
 {
-    const long n = (long)P.nx * P.ny;
-    faces_kernel<<<(int)((n + 255) / 256), 256, 0, s>>>(P, fp64_inner ? 1 : 0);
-    if (n_items <= 0) return cudaGetLastError();
-    if (fp64_inner)
-        solve_items_kernel<double><<<n_items, kSolveThreads, 0, s>>>(P, items);
-    else
-        solve_items_kernel<float><<<n_items, kSolveThreads, 0, s>>>(P, items);
+    static std::mutex mu;
+    static std::set<std::pair<const void*, int>> done;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({fn, dev})) return cudaSuccess;
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kChipSmem);
+    if (e == cudaSuccess && cluster) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) done.insert({fn, dev});
+    return e;
+}
+
+template <typename TI, bool CL, int NS>
+cudaError_t launch_chip_class(const SolveParams& P, const SolveParams* probs, const ChipLaunch& c, const int2* items,
+                              cudaStream_t s)
+{
+    cudaError_t e = chip_allow(reinterpret_cast<const void*>(&chip_kernel<TI, CL, NS>), CL);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(c.cw * c.count));
+    cfg.blockDim = dim3((unsigned)(32 * c.nw));
+    cfg.dynamicSmemBytes = (size_t)c.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)c.cw;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = CL ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, chip_kernel<TI, CL, NS>, P, probs, items + c.first);
+}
+
+template <typename TI, int NS>
+cudaError_t launch_chip_team(const SolveParams& P, const SolveParams* probs, const ChipLaunch& c, const int2* items,
+                             cudaStream_t s)
+{
+    return c.cw > 1 ? launch_chip_class<TI, true, NS>(P, probs, c, items, s)
+                    : launch_chip_class<TI, false, NS>(P, probs, c, items, s);
+}
+
+// The on-chip launches of a plan, then the global-memory one.
+cudaError_t launch_plan_solves(const SolveParams& P, const SolveParams* probs, const SolvePlan& plan,
+                               const int2* chip_items, const SolveItem* items, bool fp64_inner, cudaStream_t s)
+{
+    for (const ChipLaunch& c : plan.chip) {
+        cudaError_t e;
+        if (fp64_inner)
+            e = c.slots == 4 ? launch_chip_team<double, 4>(P, probs, c, chip_items, s)
+                             : launch_chip_team<double, 2>(P, probs, c, chip_items, s);
+        else
+            e = c.slots == 8 ? launch_chip_team<float, 8>(P, probs, c, chip_items, s)
+                             : launch_chip_team<float, 4>(P, probs, c, chip_items, s);
+        if (e != cudaSuccess) return e;
+    }
+    const int n = (int)plan.items.size();
+    if (n > 0) {
+        if (probs) {
+            if (fp64_inner) solve_batch_items_kernel<double><<<n, kSolveThreads, 0, s>>>(probs, items);
+            else solve_batch_items_kernel<float><<<n, kSolveThreads, 0, s>>>(probs, items);
+        } else {
+            if (fp64_inner) solve_items_kernel<double><<<n, kSolveThreads, 0, s>>>(P, items);
+            else solve_items_kernel<float><<<n, kSolveThreads, 0, s>>>(P, items);
+        }
+    }
     return cudaGetLastError();
 }
 
-cudaError_t launch_solve_batch_items(const SolveParams* probs, const SolveItem* items, int n_items,
-                                     bool fp64_inner, cudaStream_t s)
-{
-    if (n_items <= 0) return cudaSuccess;
-    if (fp64_inner)
-        solve_batch_items_kernel<double><<<n_items, kSolveThreads, 0, s>>>(probs, items);
-    else
-        solve_batch_items_kernel<float><<<n_items, kSolveThreads, 0, s>>>(probs, items);
-    return cudaGetLastError();
-}
+}  // namespace
 
 cudaError_t launch_faces_batch(const SolveParams* probs, const int32_t* blk_off, int n, int total_blocks,
                                bool fp64_inner, cudaStream_t s)
@@ -922,32 +964,26 @@ cudaError_t launch_faces(const SolveParams& P, bool fp64_inner, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_solve_batch(const SolveParams* probs, const int32_t* sub_off, int n, int total_subs,
-                               bool fp64_inner, cudaStream_t s, bool any_be, bool any_fe, const int2* order)
+cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const int2* chip_items,
+                               const SolveItem* items, bool fp64_inner, bool any_fe, const int2* order, int total_subs,
+                               cudaStream_t s)
 {
-    if (total_subs <= 0) return cudaSuccess;
-    if (any_be) {
-        if (fp64_inner)
-            solve_batch_kernel<double><<<total_subs, kSolveThreads, 0, s>>>(probs, sub_off, order, n);
-        else
-            solve_batch_kernel<float><<<total_subs, kSolveThreads, 0, s>>>(probs, sub_off, order, n);
-    }
-    if (any_fe) fe_batch_kernel<<<total_subs, kSolveThreads, 0, s>>>(probs, sub_off, order, n);
+    const cudaError_t e = launch_plan_solves(SolveParams{}, probs, plan, chip_items, items, fp64_inner, s);
+    if (e != cudaSuccess) return e;
+    if (any_fe && total_subs > 0) fe_batch_kernel<<<total_subs, kSolveThreads, 0, s>>>(probs, order);
     return cudaGetLastError();
 }
 
-cudaError_t launch_solve(const SolveParams& P, bool fp64_inner, cudaStream_t s)
+cudaError_t launch_solve(const SolveParams& P, const SolvePlan& plan, const int2* chip_items, const SolveItem* items,
+                         bool fp64_inner, cudaStream_t s)
 {
-    const long n = (long)P.nx * P.ny;
-    faces_kernel<<<(int)((n + 255) / 256), 256, 0, s>>>(P, fp64_inner ? 1 : 0);
-    const int nsub = P.px * P.py;
-    if (P.scheme == 1)
-        fe_kernel<<<nsub, kSolveThreads, 0, s>>>(P);
-    else if (fp64_inner)
-        solve_kernel<double><<<nsub, kSolveThreads, 0, s>>>(P);
-    else
-        solve_kernel<float><<<nsub, kSolveThreads, 0, s>>>(P);
-    return cudaGetLastError();
+    const cudaError_t e = launch_faces(P, fp64_inner, s);
+    if (e != cudaSuccess) return e;
+    if (P.scheme == 1) {
+        fe_kernel<<<P.px * P.py, kSolveThreads, 0, s>>>(P);
+        return cudaGetLastError();
+    }
+    return launch_plan_solves(P, nullptr, plan, chip_items, items, fp64_inner, s);
 }
 
 }  // namespace sdd
