@@ -137,8 +137,8 @@ constexpr int kTasksPerRound = 256;
 // path, so there the count wanted is low: in FP32 2432 tasks, half the resident warps (form 1,
 // 200 x 141 nodes, 1000 paths of about 97 substeps a node: 0.91 ms against 1.41 ms unsplit; four
 // times as many tasks win 4 % more there and cost up to 8 % where paths are shorter), in FP64 608,
-// one per SM sub-partition, whose unit a few warps fill (33 x 33, 61 x 1000 paths: 0.47 ms against
-// 1.54).  FP32 paths of form 0 are the most uneven, exit after a few substeps and gain nothing
+// one per SM sub-partition, whose unit a few warps fill (33 x 33, 61 x 1000 paths: 0.20 ms against
+// 0.69), twice that where no path exits (five rings, K = 1: 0.86 ms against 0.92).  FP32 paths of form 0 are the most uneven, exit after a few substeps and gain nothing
 // (sixteen bump problems in a batch: 20.3 ms against 20.6), so they keep tp, as do compensated
 // FP32 sums, whose value depends on the grouping beyond the FP64 rounding.
 // Periodic paths all run K substeps and leave no lane idle: many tasks even out the last wave
@@ -148,7 +148,7 @@ inline int fill_task_paths(int64_t nodes, int64_t n0, int tp, bool fp64, int acc
                            int K)
 {
     if (!fp64 && (acc_mode == kAccKahan32 || (form == 0 && !periodic))) return 0;
-    int64_t want = fp64 ? 608 : 2432;
+    int64_t want = fp64 ? (periodic ? 1216 : 608) : 2432;
     int t = tp;
     if (periodic && K > 1) {
         want = 32768;
@@ -186,6 +186,7 @@ template <typename T> struct McProblem {
     uint32_t cell_bias;        // (nx + 1) * 0x4B000000 mod 2^32: see monitor_at
     float gs[2];               // FP32 Dirichlet cell location: nx - 1, ny - 1 (see monitor_at)
     uint32_t cell_last;        // nx ny - 1: the last FP32 cell record
+    T gn[2];                   // nx - 1, ny - 1
     const T* bnd;              // moving boundary: tangential boundary coordinates (null: identity)
 };
 
@@ -194,6 +195,8 @@ template <typename T>
 inline void set_grid_consts(McProblem<T>& R)
 {
     R.cell_bias = (uint32_t)(R.nx + 1) * 0x4B000000u;
+    R.gn[0] = (T)(R.nx - 1);
+    R.gn[1] = (T)(R.ny - 1);
     R.gs[0] = (float)(R.nx - 1);
     R.gs[1] = (float)(R.ny - 1);
     R.cell_last = (uint32_t)R.nx * (uint32_t)R.ny - 1u;
