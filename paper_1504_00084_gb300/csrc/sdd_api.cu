@@ -427,7 +427,7 @@ sdd_status run_solve(sdd_problem* p)
     SDD_CK(cudaEventRecord(p->solve_ev[0], p->stream));
     SDD_CK(launch_solve(S, p->plan, p->chip_items, p->solve_items, p->fp64, p->stream));
     SDD_CK(cudaEventRecord(p->solve_ev[1], p->stream));
-    p->launches += 1 + (p->prm.subdomain_scheme == 1 ? 1 : (int)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1));
+    p->launches += 1 + (int)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1);
     const int ns = p->prm.px * p->prm.py;
     std::vector<int32_t> it(ns), ou(ns), ok(ns);
     std::vector<double> rs(ns);
@@ -541,11 +541,9 @@ sdd_problem* problem_shell(const sdd_params& prm, cudaStream_t stream)
             if (m > mg) mg = m;
         }
     p->mg_stride = mg;
-    if (prm.subdomain_scheme == 0) {
-        std::vector<SolveSub> subs;
-        solve_subs(0, prm.nx, prm.ny, prm.px, prm.py, subs);
-        p->plan = solve_plan(subs, p->fp64);
-    }
+    std::vector<SolveSub> subs;
+    solve_subs(0, prm.nx, prm.ny, prm.px, prm.py, prm.subdomain_scheme, subs);
+    p->plan = solve_plan(subs, p->fp64);
     p->stats.M = p->M;
     p->stats.t = prm.t0;
     return p;

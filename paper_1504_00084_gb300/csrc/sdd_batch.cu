@@ -44,7 +44,7 @@ struct sdd_batch {
     int n = 0;
     int M = 0;                       // interface nodes of all problems
     int total_subs = 0;
-    std::vector<int32_t> node_off, sub_off;
+    std::vector<int32_t> node_off;
     int mc_grid = 1;
     int tpb = 256;                   // path-kernel threads per block (sdd_batch_tune)
     int bps = 0;                     // resident path-kernel blocks per SM (0: the register limit)
@@ -68,9 +68,7 @@ struct sdd_batch {
     SolveParams* solve_host = nullptr;
     double* t_dev = nullptr;
     double* t_host = nullptr;
-    int32_t* sub_off_dev = nullptr;
-    int2* order_dev = nullptr;       // solve CTAs: (problem, subdomain), largest subdomains first
-    SolvePlan plan;                  // how the backward-Euler subdomains are solved
+    SolvePlan plan;                  // how the subdomains are solved
     SolveItem* items_dev = nullptr;
     int2* chip_items_dev = nullptr;
     // batched per-problem launches: records (refreshed every step) and per-problem block offsets
@@ -78,7 +76,7 @@ struct sdd_batch {
     BatchRec* rec_host = nullptr;
     int32_t* blk_off_dev = nullptr;
     int total_blocks = 0;
-    bool any_moving = false;
+    int moving_nodes = 0;        // longest side of the problems with a moving boundary
     int mc_mode = -1;            // problem switches shared by every problem (launch_mc's batch_mode), or -1
     int32_t* h_n_active = nullptr;
     // graph
@@ -240,8 +238,8 @@ sdd_status record_step(sdd_batch* b, bool first_plan = false)
     B_CK(cudaMemcpyAsync(b->t_dev, b->t_host, sizeof(double) * b->n, cudaMemcpyHostToDevice, b->stream));
     B_CK(cudaMemcpyAsync(b->rec_dev, b->rec_host, sizeof(BatchRec) * b->n, cudaMemcpyHostToDevice, b->stream));
     // monitor, packing and moving boundary of every problem, then the estimator shifts: one launch each
-    B_CK(launch_prep_batch(b->rec_dev, b->blk_off_dev, b->n, b->total_blocks, b->fp64, b->any_moving, b->stream));
-    launches += 2 + (b->any_moving ? 1 : 0);
+    B_CK(launch_prep_batch(b->rec_dev, b->blk_off_dev, b->n, b->total_blocks, b->fp64, b->moving_nodes, b->stream));
+    launches += 2 + (b->moving_nodes > 0 ? 1 : 0);
     if (b->M > 0) {
         B_CK(launch_shift_batch(b->rec_dev, b->node_prob, b->M, b->shift, b->stream));
         launches += 1;
@@ -321,13 +319,10 @@ sdd_status record_step(sdd_batch* b, bool first_plan = false)
     launches += 1 + (b->M > 0 ? 1 : 0);
     B_CK(launch_faces_batch(b->solve_dev, b->blk_off_dev, b->n, b->total_blocks, fp64_inner, b->stream));
     launches += 1;
-    bool any_fe = false;
-    for (const sdd_problem* p : b->probs) any_fe = any_fe || p->prm.subdomain_scheme == 1;
     B_CK(cudaEventRecord(b->sev0, b->stream));
-    B_CK(launch_solve_batch(b->solve_dev, b->plan, b->chip_items_dev, b->items_dev, fp64_inner, any_fe, b->order_dev,
-                            b->total_subs, b->stream));
+    B_CK(launch_solve_batch(b->solve_dev, b->plan, b->chip_items_dev, b->items_dev, fp64_inner, b->stream));
     B_CK(cudaEventRecord(b->sev1, b->stream));
-    launches += (int64_t)b->plan.chip.size() + (b->plan.items.empty() ? 0 : 1) + (any_fe ? 1 : 0);
+    launches += (int64_t)b->plan.chip.size() + (b->plan.items.empty() ? 0 : 1);
     B_CK(launch_copy_back_batch(b->rec_dev, b->blk_off_dev, b->n, b->total_blocks, b->stream));
     launches += 1;
     b->launches_per_step = launches;
@@ -374,7 +369,6 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
     b->task_paths = problems[0]->task_paths;
     std::vector<int32_t> node_prob, node_role;
     bool sampled_any = false;
-    b->sub_off.push_back(0);
     for (int i = 0; i < n; ++i) {
         b->node_off.push_back(b->M);
         b->M += problems[i]->M;
@@ -382,7 +376,6 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
         node_role.insert(node_role.end(), problems[i]->h_role.begin(), problems[i]->h_role.end());
         sampled_any = sampled_any || problems[i]->n_interp > 0;
         b->total_subs += problems[i]->prm.px * problems[i]->prm.py;
-        b->sub_off.push_back(b->total_subs);
     }
     const size_t M = (size_t)b->M + 1;
     const size_t rec = b->fp64 ? sizeof(McProblem<double>) : sizeof(McProblem<float>);
@@ -395,9 +388,7 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
     ALLOC(b->task_off, (M + 1) * 8); ALLOC(b->node_of, M * 4); ALLOC(b->task_len, M * 4); ALLOC(b->n_active, 16);
     ALLOC(b->task_counter, 16); ALLOC(b->slots, M * kSlotsPerNode * sizeof(TaskSlot));
     ALLOC(b->mcprob_dev, rec * n); ALLOC(b->solve_dev, sizeof(SolveParams) * n); ALLOC(b->t_dev, 8 * n);
-    ALLOC(b->sub_off_dev, 4 * (n + 1));
     ALLOC(b->rec_dev, sizeof(BatchRec) * n); ALLOC(b->blk_off_dev, 4 * (n + 1));
-    ALLOC(b->order_dev, sizeof(int2) * (size_t)(b->total_subs > 0 ? b->total_subs : 1));
     if (sampled_any) ALLOC(b->node_role, M * 4);
     HALLOC(b->mcprob_host, rec * n); HALLOC(b->solve_host, sizeof(SolveParams) * n); HALLOC(b->t_host, 8 * n);
     HALLOC(b->h_n_active, 32); HALLOC(b->rec_host, sizeof(BatchRec) * n);
@@ -412,13 +403,12 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
         e = cudaEventCreateWithFlags(&b->count_ev[k], cudaEventDisableTiming);
     if (e == cudaSuccess && b->M > 0)
         e = cudaMemcpy(b->node_prob, node_prob.data(), 4 * (size_t)b->M, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(b->sub_off_dev, b->sub_off.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
         std::vector<int32_t> blk_off(1, 0);
         for (int i = 0; i < n; ++i) {
             blk_off.push_back(blk_off.back() + batch_blocks((long)problems[i]->prm.nx * problems[i]->prm.ny));
-            b->any_moving = b->any_moving || (problems[i]->prm.moving_boundary && !problems[i]->prm.periodic);
+            if (problems[i]->prm.moving_boundary && !problems[i]->prm.periodic)
+                b->moving_nodes = std::max(b->moving_nodes, std::max(problems[i]->prm.nx, problems[i]->prm.ny));
         }
         b->total_blocks = blk_off.back();
         e = cudaMemcpy(b->blk_off_dev, blk_off.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice);
@@ -430,29 +420,12 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
         }
     }
     if (e == cudaSuccess && b->total_subs > 0) {
-        // longest-first: subdomains by interior size, descending (ties in problem, subdomain order)
-        std::vector<std::pair<int64_t, int2>> subs;
+        std::vector<SolveSub> subs;
         for (int i = 0; i < n; ++i) {
             const sdd_params& q = problems[i]->prm;
-            for (int k = 0; k < q.px * q.py; ++k) {
-                const int I = k % q.px, J = k / q.px;
-                const int64_t wi = split_line(I + 1, q.nx, q.px) - split_line(I, q.nx, q.px) - 1;
-                const int64_t wj = split_line(J + 1, q.ny, q.py) - split_line(J, q.ny, q.py) - 1;
-                subs.push_back({wi * wj, make_int2(i, k)});
-            }
+            solve_subs(i, q.nx, q.ny, q.px, q.py, q.subdomain_scheme, subs);
         }
-        std::stable_sort(subs.begin(), subs.end(), [](const std::pair<int64_t, int2>& a,
-                                                      const std::pair<int64_t, int2>& c) { return a.first > c.first; });
-        std::vector<int2> order;
-        for (const auto& v : subs) order.push_back(v.second);
-        e = cudaMemcpy(b->order_dev, order.data(), sizeof(int2) * order.size(), cudaMemcpyHostToDevice);
-        // backward-Euler subdomains only: forward-Euler problems run in their own kernel
-        std::vector<SolveSub> be;
-        for (int i = 0; i < n; ++i) {
-            const sdd_params& q = problems[i]->prm;
-            if (q.subdomain_scheme == 0) solve_subs(i, q.nx, q.ny, q.px, q.py, be);
-        }
-        b->plan = solve_plan(be, b->fp64);
+        b->plan = solve_plan(subs, b->fp64);
         if (e == cudaSuccess && !b->plan.items.empty()) {
             e = b->dalloc(&b->items_dev, sizeof(SolveItem) * b->plan.items.size());
             if (e == cudaSuccess)

@@ -922,6 +922,195 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ So
     chip_body<TI, CL, NS>(sp, it.y, L, &scal, chip_sm);
 }
 
+// ---- forward Euler on chip ----------------------------------------------------------------
+// The paper's local solver (fe_body's substeps) with the iterate in shared memory and each thread's
+// nodes, with their weights c_nb / (S d), in registers; a subdomain is split by rows over a cluster
+// whose edge rows are written to the neighbours' halo copies.  A substep is 18 FP64 operations a
+// node (fe_body: 48 with its divisions) and a barrier; the FP64 unit bounds it until a CTA has few
+// nodes, then the barrier.  Every node computes the same operations in any team, and the team is
+// chosen by how many subdomains the launch has.  15 subdomains of 65 x 27, 60 substeps: 1.54 ms from
+// global memory by a CTA each, 0.23 ms by clusters of eight.
+constexpr int kFeThreads = 512, kFeSlots = 4;
+__host__ __device__ inline int fe_chip_bytes(int ni, int nj, int cw)
+{
+    return 2 * ((nj + cw - 1) / cw + 2) * (ni + 2) * 16 + 128;
+}
+
+template <bool CL>
+__device__ __forceinline__ void fe_chip_body(const SolveParams& P, int sub, char* sm)
+{
+    Chip<CL> T;
+    T.sm = sm;
+    T.rank = 0; T.cw = 1; T.dn = T.up = nullptr;
+    if constexpr (CL) {
+        cg::cluster_group cl = cg::this_cluster();
+        T.rank = (int)cl.block_rank();
+        T.cw = (int)cl.num_blocks();
+        if (T.rank > 0) T.dn = cl.map_shared_rank(sm, T.rank - 1);
+        if (T.rank + 1 < T.cw) T.up = cl.map_shared_rank(sm, T.rank + 1);
+    }
+    const int tid = threadIdx.x, nx = P.nx;
+    const int I = sub % P.px, J = sub / P.px;
+    const int i0 = split_line(I, nx, P.px), i1 = split_line(I + 1, nx, P.px);
+    const int j0 = split_line(J, P.ny, P.py), j1 = split_line(J + 1, P.ny, P.py);
+    const int ni = i1 - i0 - 1, nj = j1 - j0 - 1;
+    if (ni <= 0 || nj <= 0) {  // no interior (a team of one CTA)
+        if (tid == 0) {
+            P.stat_iters[sub] = 1; P.stat_outer[sub] = 0; P.stat_ok[sub] = 1; P.stat_res[sub] = 0.0;
+        }
+        return;
+    }
+    const int r0 = (int)((long)T.rank * nj / T.cw), r1 = (int)((long)(T.rank + 1) * nj / T.cw), nr = r1 - r0;
+    const int below = T.rank > 0 ? r0 - (int)((long)(T.rank - 1) * nj / T.cw) : 0;
+    const int rows = (nj + T.cw - 1) / T.cw, W = ni + 2;
+    double* red = reinterpret_cast<double*>(sm);                // 16: warps' maxima, then CTAs'
+    double2* buf = reinterpret_cast<double2*>(sm + 128);        // two buffers of (rows + 2) x W
+    const int cells = (rows + 2) * W;
+    auto dP = [&](long id) -> double { return P.form == 0 ? 1.0 : P.om64[id]; };
+    // own nodes: place in a buffer, coefficients, value
+    int at_[kFeSlots];
+    double aE[kFeSlots], aW[kFeSlots], aN[kFeSlots], aS[kFeSlots];
+    double2 x[kFeSlots];
+    double cmax = 0.0;
+#pragma unroll
+    for (int s = 0; s < kFeSlots; ++s) {
+        const int k = tid + s * kFeThreads;
+        at_[s] = -1;
+        if (k >= nr * ni) continue;
+        const int jl = k / ni, i = k % ni;
+        const long id = (long)(j0 + 1 + r0 + jl) * nx + (i0 + 1 + i);
+        at_[s] = (jl + 1) * W + i + 1;
+        aE[s] = P.ce64[id]; aW[s] = P.ce64[id - 1]; aN[s] = P.cn64[id]; aS[s] = P.cn64[id - nx];
+        x[s] = make_double2(P.xcur[id], P.ycur[id]);
+        const double c = __dadd_rn(__dadd_rn(__dadd_rn(aE[s], aW[s]), aN[s]), aS[s]);
+        cmax = fmax(cmax, P.form == 0 ? c : __ddiv_rn(c, P.om64[id]));
+    }
+    // largest over the team (the same value in any order)
+    for (int o = 16; o > 0; o >>= 1) cmax = fmax(cmax, __shfl_xor_sync(kFull, cmax, o));
+    if ((tid & 31) == 0) red[tid >> 5] = cmax;
+    __syncthreads();
+    cmax = red[0];
+    for (int w = 1; w < kFeThreads / 32; ++w) cmax = fmax(cmax, red[w]);
+    if constexpr (CL) {
+        cg::this_cluster().sync();  // every CTA has read its warps' maxima
+        if (tid < T.cw) cg::this_cluster().map_shared_rank(red, tid)[T.rank] = cmax;  // 8 CTAs at most
+        cg::this_cluster().sync();
+        cmax = red[0];
+        for (int r = 1; r < T.cw; ++r) cmax = fmax(cmax, red[r]);
+    }
+    const double Sd = ceil(cmax) < 1.0 ? 1.0 : ceil(cmax);
+    const bool solve = Sd <= (double)P.fe_max_substeps;
+    const int S = solve ? (int)Sd : 0;
+    // the rim cells of this CTA: the columns beside its rows, and the rows below the first and above the
+    // last CTA's; cell k's place and node
+    const int nrim = 2 * nr + (T.rank == 0 ? ni : 0) + (T.rank == T.cw - 1 ? ni : 0);
+    auto rim = [&](int k, int& place, long& id) {
+        int jl, i;
+        if (k < 2 * nr) { jl = k >> 1; i = (k & 1) ? ni : -1; }
+        else {
+            k -= 2 * nr;
+            const bool low = T.rank == 0 && k < ni;
+            if (T.rank == 0 && !low) k -= ni;
+            jl = low ? -1 : nr;
+            i = k;
+        }
+        place = (jl + 1) * W + i + 1;
+        id = (long)(j0 + 1 + r0 + jl) * nx + (i0 + 1 + i);
+    };
+    int rim_at = -1;             // the thread's first rim cell in registers, further ones from memory
+    double2 rim_x = make_double2(0.0, 0.0), rim_d = rim_x;
+    if (tid < nrim) {
+        long id;
+        rim(tid, rim_at, id);
+        rim_x = make_double2(P.xcur[id], P.ycur[id]);
+        rim_d = make_double2(__dsub_rn(P.xnew[id], rim_x.x), __dsub_rn(P.ynew[id], rim_x.y));
+    }
+    auto write_rim = [&](double2* b, double f) {  // x^n + f (x^{n+1} - x^n)
+        if (rim_at >= 0)
+            b[rim_at] = make_double2(__dadd_rn(rim_x.x, __dmul_rn(f, rim_d.x)), __dadd_rn(rim_x.y, __dmul_rn(f, rim_d.y)));
+        for (int k = tid + kFeThreads; k < nrim; k += kFeThreads) {
+            int place;
+            long id;
+            rim(k, place, id);
+            const double px = P.xcur[id], py = P.ycur[id];
+            b[place] = make_double2(__dadd_rn(px, __dmul_rn(f, __dsub_rn(P.xnew[id], px))),
+                                    __dadd_rn(py, __dmul_rn(f, __dsub_rn(P.ynew[id], py))));
+        }
+    };
+    auto write_node = [&](int which, int place, double2 v) {
+        buf[which * cells + place] = v;
+        if constexpr (CL) {
+            if (T.rank > 0 && place < 2 * W) at<double2>(T.dn, 128)[which * cells + place + below * W] = v;
+            if (T.rank + 1 < T.cw && place >= nr * W) at<double2>(T.up, 128)[which * cells + place - nr * W] = v;
+        }
+    };
+#pragma unroll
+    for (int s = 0; s < kFeSlots; ++s) {
+        if (at_[s] < 0) continue;
+        const int k = tid + s * kFeThreads;
+        const long id = (long)(j0 + 1 + r0 + k / ni) * nx + (i0 + 1 + k % ni);
+        const double w = __ddiv_rn(1.0, __dmul_rn(Sd, dP(id)));
+        aE[s] *= w; aW[s] *= w; aN[s] *= w; aS[s] *= w;
+        write_node(0, at_[s], x[s]);
+    }
+    write_rim(buf, 0.0);
+    T.sync(1);
+#pragma unroll 1
+    for (int m = 0; m < S; ++m) {
+        const double2* b = buf + (m & 1) * cells;
+        const int to = (m + 1) & 1;
+#pragma unroll
+        for (int s = 0; s < kFeSlots; ++s) {
+            if (at_[s] < 0) continue;
+            const double2 e = b[at_[s] + 1], w = b[at_[s] - 1], n = b[at_[s] + W], so = b[at_[s] - W];
+            const double dx = fma(aS[s], so.x - x[s].x, fma(aN[s], n.x - x[s].x, fma(aW[s], w.x - x[s].x, aE[s] * (e.x - x[s].x))));
+            const double dy = fma(aS[s], so.y - x[s].y, fma(aN[s], n.y - x[s].y, fma(aW[s], w.y - x[s].y, aE[s] * (e.y - x[s].y))));
+            x[s].x += dx;
+            x[s].y += dy;
+            write_node(to, at_[s], x[s]);
+        }
+        write_rim(buf + to * cells, (double)(m + 1) / Sd);
+        T.sync(1);
+    }
+#pragma unroll
+    for (int s = 0; s < kFeSlots; ++s) {
+        if (at_[s] < 0) continue;
+        const int k = tid + s * kFeThreads;
+        const long id = (long)(j0 + 1 + r0 + k / ni) * nx + (i0 + 1 + k % ni);
+        P.xnew[id] = x[s].x;  // x^n where the subdomain needs more substeps than allowed
+        P.ynew[id] = x[s].y;
+    }
+    if (T.rank == 0 && tid == 0) {
+        P.stat_iters[sub] = S; P.stat_outer[sub] = 0; P.stat_ok[sub] = solve ? 1 : 0; P.stat_res[sub] = 0.0;
+    }
+    if constexpr (CL) cg::this_cluster().sync();  // no CTA leaves while another may still write to it
+}
+
+template <bool CL>
+__global__ void __launch_bounds__(kFeThreads, 1) fe_chip_kernel(const __grid_constant__ SolveParams P, const SolveParams* probs,
+                                                                const int2* items)
+{
+    extern __shared__ __align__(16) char chip_sm[];
+    __shared__ SolveParams sp;
+    int team = blockIdx.x;
+    if constexpr (CL) team /= (int)cg::this_cluster().num_blocks();
+    const int2 it = items[team];
+    if (threadIdx.x == 0) sp = probs ? probs[it.x] : P;
+    __syncthreads();
+    fe_chip_body<CL>(sp, it.y, chip_sm);
+}
+
+// CTAs of the smallest team that holds a subdomain of ni x nj nodes (0: none of up to eight does).
+inline int fe_chip_team(int ni, int nj)
+{
+    if (ni <= 0 || nj <= 0) return 1;
+    for (int cw = 1; cw <= 8; cw *= 2)
+        if (nj >= cw && (int64_t)((nj + cw - 1) / cw) * ni <= kFeThreads * kFeSlots && ni <= 4096 &&
+            fe_chip_bytes(ni, nj, cw) <= kChipSmem)
+            return cw;
+    return 0;
+}
+
 // Team of a subdomain of ni x nj interior nodes: CTAs (0: it does not fit), warps per CTA, slots of
 // its kernel, dynamic shared memory.  The fewest CTAs that hold it -- a cluster barrier costs about a
 // microsecond, ten times a CTA's -- as a function of the size alone, so that a subdomain gives the

@@ -339,12 +339,14 @@ struct SolveItem {
     int32_t prob, sub, width, pad;
 };
 
-// A subdomain to be solved by backward Euler: subdomain `sub` of problem `prob`, ni x nj interior nodes.
+// A subdomain to be solved: subdomain `sub` of problem `prob`, ni x nj interior nodes, by backward (0) or
+// forward (1) Euler.
 struct SolveSub {
-    int32_t prob, sub, ni, nj;
+    int32_t prob, sub, ni, nj, scheme;
 };
-// One launch of the on-chip solve kernel (sdd_chip.cuh): `count` subdomains from items[first] on, each
-// by cw CTAs of nw warps, `slots` nodes a thread, with smem bytes of dynamic shared memory.
+// One launch of an on-chip solve kernel (sdd_chip.cuh): `count` subdomains from items[first] on, each
+// by cw CTAs of nw warps, `slots` nodes a thread, with smem bytes of dynamic shared memory.  slots 0:
+// forward Euler (cw 0: from global memory).
 struct ChipLaunch {
     int cw, nw, slots, smem, first, count;
 };
@@ -359,7 +361,7 @@ struct SolvePlan {
 // The plan of the subdomains of one problem's split (solve_subs), or of several problems'.
 SolvePlan solve_plan(std::vector<SolveSub> subs, bool fp64);
 // Subdomains of an nx x ny grid split px x py, appended to `subs` as problem `prob`.
-void solve_subs(int prob, int nx, int ny, int px, int py, std::vector<SolveSub>& subs);
+void solve_subs(int prob, int nx, int ny, int px, int py, int scheme, std::vector<SolveSub>& subs);
 
 // Multigrid hierarchy of an n x m subdomain interior: the coarse grid keeps the nodes of odd
 // index, (n - 1) / 2 of them for odd n and n / 2 for even n (then the last coarse node lies one
@@ -431,19 +433,18 @@ cudaError_t launch_faces(const SolveParams& P, bool fp64_inner, cudaStream_t s);
 // Batched launches of a batch step (blk_off: per-problem block offsets of grid-sized work, n + 1
 // entries, blocks of 256 threads as batch_blocks gives them; node work over the concatenated nodes).
 int batch_blocks(long n_nodes);
+// moving_nodes: the longest side of the problems with a moving boundary (0: none)
 cudaError_t launch_prep_batch(const BatchRec* R, const int32_t* blk_off, int n, int total_blocks, bool fp64,
-                              bool any_moving, cudaStream_t s);
+                              int moving_nodes, cudaStream_t s);
 cudaError_t launch_shift_batch(const BatchRec* R, const int32_t* node_prob, int M, double* shift, cudaStream_t s);
 cudaError_t launch_scatter_batch(const BatchRec* R, const int32_t* blk_off, int n, int total_blocks,
                                  const int32_t* node_prob, int M, const double* est, cudaStream_t s);
 cudaError_t launch_copy_back_batch(const BatchRec* R, const int32_t* blk_off, int n, int total_blocks, cudaStream_t s);
 cudaError_t launch_faces_batch(const SolveParams* probs, const int32_t* blk_off, int n, int total_blocks,
                                bool fp64_inner, cudaStream_t s);
-// Backward-Euler solves of a batch (plan's items in device memory), then its forward-Euler problems
-// (any_fe; order: (problem, subdomain) of each CTA).
+// Subdomain solves of a batch (plan's items in device memory).
 cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const int2* chip_items,
-                               const SolveItem* items, bool fp64_inner, bool any_fe, const int2* order, int total_subs,
-                               cudaStream_t s);
+                               const SolveItem* items, bool fp64_inner, cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, const uint32_t* key, int64_t n, uint32_t* out,
                           cudaStream_t s);
 cudaError_t launch_unit_math(const uint32_t* w, int64_t n, float* out, cudaStream_t s);

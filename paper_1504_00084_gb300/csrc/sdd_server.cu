@@ -398,7 +398,7 @@ sdd_status finish(sdd_server* s, Request* r)
     S.mg = p->mg; S.mg_stride = p->mg_stride;
     S.stat_iters = p->st_iters; S.stat_outer = p->st_outer; S.stat_ok = p->st_ok; S.stat_res = p->st_res;
     S_CK(launch_solve(S, p->plan, p->chip_items, p->solve_items, s->fp64, s->fin));
-    s->st.kernel_launches += 1 + (S.scheme == 1 ? 1 : (int64_t)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1));
+    s->st.kernel_launches += 1 + (int64_t)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1);
     S_CK(cudaEventRecord(r->done_ev, s->fin));
     r->state = kFinishing;
     return SDD_OK;

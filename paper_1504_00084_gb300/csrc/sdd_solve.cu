@@ -44,6 +44,7 @@ namespace {
 constexpr int kSolveThreads = 512;
 constexpr int kSolveMinBlocks = 1024 / kSolveThreads;
 constexpr int kMaxOuter = 12;
+constexpr int kSms = 152;  // of a GB300
 constexpr int kCoarseSweeps = 4;  // symmetric Gauss-Seidel sweeps on the coarsest level
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -751,22 +752,17 @@ __device__ __forceinline__ void solve_body(const Team<CW>& tm, const SolveParams
 template <typename TI, int CW>
 __device__ SDD_SOLVE_SUB_ATTR void solve_sub(const Team<CW> tm, const SolveParams& P, int sub, double* sh);
 
-__global__ void __launch_bounds__(kSolveThreads) fe_kernel(const __grid_constant__ SolveParams P)
-{
-    __shared__ double sh[40];
-    fe_body(P, blockIdx.x, sh);
-}
-
-// Batched forward-Euler subdomains, order[b] = (problem, subdomain) of CTA b (CTAs of backward-Euler
-// problems return at once).
-__global__ void __launch_bounds__(kSolveThreads) fe_batch_kernel(const SolveParams* probs, const int2* order)
+// Forward-Euler subdomains from global memory, items[b] = (problem, subdomain) of CTA b (probs null: the
+// problem P).
+__global__ void __launch_bounds__(kSolveThreads) fe_kernel(const __grid_constant__ SolveParams P, const SolveParams* probs,
+                                                           const int2* items)
 {
     __shared__ double sh[40];
     __shared__ SolveParams sp;
-    const int2 o = order[blockIdx.x];
-    if (threadIdx.x == 0) sp = probs[o.x];
+    const int2 o = items[blockIdx.x];
+    if (threadIdx.x == 0) sp = probs ? probs[o.x] : P;
     __syncthreads();
-    if (sp.scheme == 1) fe_body(sp, o.y, sh);
+    fe_body(sp, o.y, sh);
 }
 
 // The solve of one subdomain, called by every solve kernel.  Inlined into each kernel (measured
@@ -823,12 +819,12 @@ __global__ void __cluster_dims__(kCoopWidth, 1, 1) __launch_bounds__(kSolveThrea
 
 #include "sdd_chip.cuh"
 
-void solve_subs(int prob, int nx, int ny, int px, int py, std::vector<SolveSub>& subs)
+void solve_subs(int prob, int nx, int ny, int px, int py, int scheme, std::vector<SolveSub>& subs)
 {
     for (int k = 0; k < px * py; ++k) {
         const int I = k % px, J = k / px;
         subs.push_back(SolveSub{prob, k, split_line(I + 1, nx, px) - split_line(I, nx, px) - 1,
-                                split_line(J + 1, ny, py) - split_line(J, ny, py) - 1});
+                                split_line(J + 1, ny, py) - split_line(J, ny, py) - 1, scheme});
     }
 }
 
@@ -841,10 +837,25 @@ SolvePlan solve_plan(std::vector<SolveSub> subs, bool fp64)
     SolvePlan plan;
     std::vector<std::pair<ChipLaunch, std::vector<int2>>> classes;
     std::vector<SolveItem> pend;  // subdomains of one CTA each, waiting to fill a cluster
+    // forward Euler: its results do not depend on the team, so few subdomains get more CTAs each, as
+    // long as all run at once and every CTA has a few rows
+    int64_t n_fe = 0;
+    for (const SolveSub& v : subs) n_fe += v.scheme == 1 ? 1 : 0;
     for (const SolveSub& v : subs) {
         ChipLaunch c{};
-        chip_team(v.ni, v.nj, fp64, &c);
-        if (c.cw > 0) {
+        if (v.scheme == 1) {
+            c.cw = fe_chip_team(v.ni, v.nj);
+            if (c.cw > 0 && v.ni > 0 && v.nj > 0) {
+                while (c.cw < 8 && 2 * c.cw * n_fe <= kSms && v.nj >= 6 * c.cw) c.cw *= 2;
+                c.smem = fe_chip_bytes(v.ni, v.nj, c.cw);
+            } else if (c.cw > 0) {
+                c.smem = 1024;
+            }
+            c.nw = kFeThreads / 32;
+        } else {
+            chip_team(v.ni, v.nj, fp64, &c);
+        }
+        if (c.cw > 0 || v.scheme == 1) {
             size_t k = 0;
             while (k < classes.size() && (classes[k].first.cw != c.cw || classes[k].first.nw != c.nw ||
                                           classes[k].first.slots != c.slots)) ++k;
@@ -893,11 +904,12 @@ cudaError_t chip_allow(const void* fn, bool cluster)
     return e;
 }
 
-template <typename TI, bool CL, int NS>
-cudaError_t launch_chip_class(const SolveParams& P, const SolveParams* probs, const ChipLaunch& c, const int2* items,
-                              cudaStream_t s)
+typedef void (*ChipKernel)(const SolveParams, const SolveParams*, const int2*);
+
+cudaError_t launch_chip_class(ChipKernel fn, bool cluster, const SolveParams& P, const SolveParams* probs,
+                              const ChipLaunch& c, const int2* items, cudaStream_t s)
 {
-    cudaError_t e = chip_allow(reinterpret_cast<const void*>(&chip_kernel<TI, CL, NS>), CL);
+    cudaError_t e = chip_allow(reinterpret_cast<const void*>(fn), cluster);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(c.cw * c.count));
@@ -909,16 +921,16 @@ cudaError_t launch_chip_class(const SolveParams& P, const SolveParams* probs, co
     at[0].val.clusterDim.x = (unsigned)c.cw;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = CL ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, chip_kernel<TI, CL, NS>, P, probs, items + c.first);
+    cfg.numAttrs = cluster ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, P, probs, items + c.first);
 }
 
 template <typename TI, int NS>
 cudaError_t launch_chip_team(const SolveParams& P, const SolveParams* probs, const ChipLaunch& c, const int2* items,
                              cudaStream_t s)
 {
-    return c.cw > 1 ? launch_chip_class<TI, true, NS>(P, probs, c, items, s)
-                    : launch_chip_class<TI, false, NS>(P, probs, c, items, s);
+    return c.cw > 1 ? launch_chip_class(chip_kernel<TI, true, NS>, true, P, probs, c, items, s)
+                    : launch_chip_class(chip_kernel<TI, false, NS>, false, P, probs, c, items, s);
 }
 
 // The on-chip launches of a plan, then the global-memory one.
@@ -927,7 +939,15 @@ cudaError_t launch_plan_solves(const SolveParams& P, const SolveParams* probs, c
 {
     for (const ChipLaunch& c : plan.chip) {
         cudaError_t e;
-        if (fp64_inner)
+        if (c.slots == 0) {
+            if (c.cw == 0) {
+                fe_kernel<<<c.count, kSolveThreads, 0, s>>>(P, probs, chip_items + c.first);
+                e = cudaGetLastError();
+            } else {
+                e = c.cw > 1 ? launch_chip_class(fe_chip_kernel<true>, true, P, probs, c, chip_items, s)
+                             : launch_chip_class(fe_chip_kernel<false>, false, P, probs, c, chip_items, s);
+            }
+        } else if (fp64_inner)
             e = c.slots == 4 ? launch_chip_team<double, 4>(P, probs, c, chip_items, s)
                              : launch_chip_team<double, 2>(P, probs, c, chip_items, s);
         else
@@ -965,25 +985,16 @@ cudaError_t launch_faces(const SolveParams& P, bool fp64_inner, cudaStream_t s)
 }
 
 cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const int2* chip_items,
-                               const SolveItem* items, bool fp64_inner, bool any_fe, const int2* order, int total_subs,
-                               cudaStream_t s)
+                               const SolveItem* items, bool fp64_inner, cudaStream_t s)
 {
-    const cudaError_t e = launch_plan_solves(SolveParams{}, probs, plan, chip_items, items, fp64_inner, s);
-    if (e != cudaSuccess) return e;
-    if (any_fe && total_subs > 0) fe_batch_kernel<<<total_subs, kSolveThreads, 0, s>>>(probs, order);
-    return cudaGetLastError();
+    return launch_plan_solves(SolveParams{}, probs, plan, chip_items, items, fp64_inner, s);
 }
 
 cudaError_t launch_solve(const SolveParams& P, const SolvePlan& plan, const int2* chip_items, const SolveItem* items,
                          bool fp64_inner, cudaStream_t s)
 {
     const cudaError_t e = launch_faces(P, fp64_inner, s);
-    if (e != cudaSuccess) return e;
-    if (P.scheme == 1) {
-        fe_kernel<<<P.px * P.py, kSolveThreads, 0, s>>>(P);
-        return cudaGetLastError();
-    }
-    return launch_plan_solves(P, nullptr, plan, chip_items, items, fp64_inner, s);
+    return e != cudaSuccess ? e : launch_plan_solves(P, nullptr, plan, chip_items, items, fp64_inner, s);
 }
 
 }  // namespace sdd
