@@ -1007,7 +1007,7 @@ sdd_status sdd_tune(sdd_problem* p, int32_t tune_paths_per_task, sdd_mc_config* 
             PP.task_paths = T;
             PP.task_len = p->task_len;
             PP.fill = fill_task_paths(p->M, n0, T, p->fp64, p->acc_mode,
-                                      p->prm.form, p->prm.periodic, p->prm.substeps);
+                                      p->prm.form, p->prm.periodic, p->prm.substeps, p->prm.dt / p->prm.tau);
             for (int bps = 1; bps <= p->mc_max_blocks_per_sm && ce == cudaSuccess; ++bps) {
                 float ms_min = 0.f;
                 for (int rep = 0; rep < 2 && ce == cudaSuccess; ++rep) {

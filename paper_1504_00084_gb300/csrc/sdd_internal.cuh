@@ -139,23 +139,25 @@ constexpr int kTasksPerRound = 256;
 // times as many tasks win 4 % more there and cost up to 8 % where paths are shorter), in FP64 608,
 // one per SM sub-partition, whose unit a few warps fill (33 x 33, 61 x 1000 paths: 0.20 ms against
 // 0.69), twice that where no path exits (five rings, K = 1: 0.86 ms against 0.92).  FP32 paths of form 0 are the most uneven, exit after a few substeps and gain nothing
-// (sixteen bump problems in a batch: 20.3 ms against 20.6), so they keep tp, as do compensated
-// FP32 sums, whose value depends on the grouping beyond the FP64 rounding.
-// Periodic paths all run K substeps and leave no lane idle: many tasks even out the last wave
-// (2032 x 4000 paths, K = 100: 7.8 ms against 10.2), as long as a task keeps 128 substeps a lane
-// to spread its own start and reduction over.
+// (sixteen bump problems in a batch: 20.3 ms against 20.6), so they keep tp.
+// Periodic paths all run K substeps, and most paths of form 1 do whose diffusion over the step,
+// sqrt(2 dt / tau), is below 0.15 of the square: they leave no lane idle, and many tasks even out the
+// last wave (2032 x 4000 periodic paths, K = 100: 6.2 ms against 10.2; 1521 nodes to SE 3e-4 in
+// chunks of 1e4 and 1.4e4: 27.5 against 33.5), as long as a task keeps 128 substeps a lane to spread its
+// own start and reduction over.
+// The value of compensated FP32 sums depends on the grouping beyond the FP64 rounding, by about
+// 2e-8 / sqrt(n0) of the spread; they are split in the even case from 4096 paths on.
 inline int fill_task_paths(int64_t nodes, int64_t n0, int tp, bool fp64, int acc_mode, int form, int periodic,
-                           int K)
+                           int K, double dt_over_tau)
 {
-    if (!fp64 && (acc_mode == kAccKahan32 || (form == 0 && !periodic))) return 0;
-    int64_t want = fp64 ? (periodic ? 1216 : 608) : 2432;
+    const bool even = K > 1 && (periodic || (form == 1 && dt_over_tau <= 0.01));
+    if (!fp64 && !periodic && form == 0) return 0;
+    if (!fp64 && acc_mode == kAccKahan32 && !(even && n0 >= 4096)) return 0;
+    const int64_t want = fp64 ? (periodic ? 1216 : 608) : 2432;
     int t = tp;
-    if (periodic && K > 1) {
-        want = 32768;
-        while (t > 32 && (int64_t)t * K >= 2 * 4096 && nodes * ((n0 + t - 1) / t) < want) t >>= 1;
-    } else {
-        while (t > 32 && nodes * ((n0 + t - 1) / t) < want) t >>= 1;
-    }
+    while (t > 32 && nodes * ((n0 + t - 1) / t) < want) t >>= 1;
+    if (even)
+        while (t > 32 && (int64_t)t * K >= 2 * 4096 && nodes * ((n0 + t - 1) / t) < 65536) t >>= 1;
     return t < tp ? t : 0;
 }
 

@@ -269,7 +269,7 @@ extern "C" sdd_status sdd_interface_mc_noalloc(const sdd_params* P, const double
     Buffers b{};
     // tasks of the size sdd_interface_mc uses, or of twice that and so on until their slots fit
     int task_paths = chunk_task_paths(chunk, fill_task_paths(M, P->paths_per_node, kPathsPerTask, fp64, acc_mode, P->form,
-                                                             P->periodic, P->substeps), kPathsPerTask);
+                                                             P->periodic, P->substeps, P->dt / P->tau), kPathsPerTask);
     int64_t slots = 0;
     for (;; task_paths <<= 1) {
         slots = M * ((chunk + task_paths - 1) / task_paths);

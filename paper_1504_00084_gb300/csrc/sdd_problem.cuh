@@ -33,7 +33,7 @@ struct sdd_problem {
     int fill() const
     {
         return sdd::fill_task_paths(M, prm.paths_per_node, task_paths, fp64, acc_mode,
-                                    prm.form, prm.periodic, prm.substeps);
+                                    prm.form, prm.periodic, prm.substeps, prm.dt / prm.tau);
     }
     int nsm = 1;
     bool fp64 = true;
