@@ -237,6 +237,7 @@ sdd_status run_prep(sdd_problem* p)
     P.t = p->monitor_time_fixed ? p->t_monitor : p->prm.t0 + (double)p->step * p->prm.dt;
     P.x = p->x; P.y = p->y; P.omega_in = p->omega_nodal;
     memcpy(P.params, p->mon_params, sizeof(P.params));
+    set_prep_consts(P);
     P.om64 = p->om64; P.wxi64 = p->wxi64; P.weta64 = p->weta64;
     P.mon = p->mon; P.disp = p->disp; P.bad = p->bad;
     P.moving_boundary = p->prm.moving_boundary; P.form = p->prm.form; P.r = p->prm.dt / p->prm.tau;
@@ -414,7 +415,7 @@ sdd_status run_solve(sdd_problem* p)
     p->launches += (p->prm.periodic ? 0 : 1) + (p->M > 0 ? 1 : 0);
     SolveParams S{};
     S.nx = p->prm.nx; S.ny = p->prm.ny; S.px = p->prm.px; S.py = p->prm.py; S.form = p->prm.form;
-    S.r = p->prm.dt / p->prm.tau; S.rtol = p->prm.solve_rtol; S.max_iter = p->prm.solve_max_iter;
+    S.r = p->prm.dt / p->prm.tau; set_face_consts(S); S.rtol = p->prm.solve_rtol; S.max_iter = p->prm.solve_max_iter;
     S.scheme = p->prm.subdomain_scheme;
     S.fe_max_substeps = p->prm.fe_max_substeps > 0 ? p->prm.fe_max_substeps : (1 << 16);
     S.om64 = p->om64; S.xcur = p->x; S.ycur = p->y; S.xnew = p->xn; S.ynew = p->yn;

@@ -74,8 +74,8 @@ struct sdd_batch {
     // batched per-problem launches: records (refreshed every step) and per-problem block offsets
     BatchRec* rec_dev = nullptr;
     BatchRec* rec_host = nullptr;
-    int32_t* blk_off_dev = nullptr;
-    int total_blocks = 0;
+    int32_t *blk_off_dev = nullptr, *tile_off_dev = nullptr;
+    int total_blocks = 0, total_tiles = 0;
     int moving_nodes = 0;        // longest side of the problems with a moving boundary
     int mc_mode = -1;            // problem switches shared by every problem (launch_mc's batch_mode), or -1
     int32_t* h_n_active = nullptr;
@@ -144,7 +144,7 @@ SolveParams solve_params(const sdd_problem* p)
 {
     SolveParams S{};
     S.nx = p->prm.nx; S.ny = p->prm.ny; S.px = p->prm.px; S.py = p->prm.py; S.form = p->prm.form;
-    S.r = p->prm.dt / p->prm.tau; S.rtol = p->prm.solve_rtol; S.max_iter = p->prm.solve_max_iter;
+    S.r = p->prm.dt / p->prm.tau; set_face_consts(S); S.rtol = p->prm.solve_rtol; S.max_iter = p->prm.solve_max_iter;
     S.scheme = p->prm.subdomain_scheme;
     S.fe_max_substeps = p->prm.fe_max_substeps > 0 ? p->prm.fe_max_substeps : (1 << 16);
     S.om64 = p->om64; S.xcur = p->x; S.ycur = p->y; S.xnew = p->xn; S.ynew = p->yn;
@@ -180,6 +180,7 @@ void refresh_records(sdd_batch* b)
         P.Lx = p->prm.Lx; P.Ly = p->prm.Ly; P.t = 0.0; P.t_dev = b->t_dev + i;
         P.x = p->x; P.y = p->y; P.omega_in = p->omega_nodal;
         memcpy(P.params, p->mon_params, sizeof(P.params));
+        set_prep_consts(P);
         P.om64 = p->om64; P.wxi64 = p->wxi64; P.weta64 = p->weta64; P.mon = p->mon; P.disp = p->disp;
         P.bad = p->bad;
         P.moving_boundary = p->prm.moving_boundary; P.form = p->prm.form; P.r = p->prm.dt / p->prm.tau;
@@ -238,7 +239,8 @@ sdd_status record_step(sdd_batch* b, bool first_plan = false)
     B_CK(cudaMemcpyAsync(b->t_dev, b->t_host, sizeof(double) * b->n, cudaMemcpyHostToDevice, b->stream));
     B_CK(cudaMemcpyAsync(b->rec_dev, b->rec_host, sizeof(BatchRec) * b->n, cudaMemcpyHostToDevice, b->stream));
     // monitor, packing and moving boundary of every problem, then the estimator shifts: one launch each
-    B_CK(launch_prep_batch(b->rec_dev, b->blk_off_dev, b->n, b->total_blocks, b->fp64, b->moving_nodes, b->stream));
+    B_CK(launch_prep_batch(b->rec_dev, b->blk_off_dev, b->tile_off_dev, b->n, b->total_blocks, b->total_tiles, b->fp64,
+                           b->moving_nodes, b->stream));
     launches += 2 + (b->moving_nodes > 0 ? 1 : 0);
     if (b->M > 0) {
         B_CK(launch_shift_batch(b->rec_dev, b->node_prob, b->M, b->shift, b->stream));
@@ -388,7 +390,7 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
     ALLOC(b->task_off, (M + 1) * 8); ALLOC(b->node_of, M * 4); ALLOC(b->task_len, M * 4); ALLOC(b->n_active, 16);
     ALLOC(b->task_counter, 16); ALLOC(b->slots, M * kSlotsPerNode * sizeof(TaskSlot));
     ALLOC(b->mcprob_dev, rec * n); ALLOC(b->solve_dev, sizeof(SolveParams) * n); ALLOC(b->t_dev, 8 * n);
-    ALLOC(b->rec_dev, sizeof(BatchRec) * n); ALLOC(b->blk_off_dev, 4 * (n + 1));
+    ALLOC(b->rec_dev, sizeof(BatchRec) * n); ALLOC(b->blk_off_dev, 4 * (n + 1)); ALLOC(b->tile_off_dev, 4 * (n + 1));
     if (sampled_any) ALLOC(b->node_role, M * 4);
     HALLOC(b->mcprob_host, rec * n); HALLOC(b->solve_host, sizeof(SolveParams) * n); HALLOC(b->t_host, 8 * n);
     HALLOC(b->h_n_active, 32); HALLOC(b->rec_host, sizeof(BatchRec) * n);
@@ -404,14 +406,18 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
     if (e == cudaSuccess && b->M > 0)
         e = cudaMemcpy(b->node_prob, node_prob.data(), 4 * (size_t)b->M, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
-        std::vector<int32_t> blk_off(1, 0);
+        std::vector<int32_t> blk_off(1, 0), tile_off(1, 0);
         for (int i = 0; i < n; ++i) {
             blk_off.push_back(blk_off.back() + batch_blocks((long)problems[i]->prm.nx * problems[i]->prm.ny));
+            tile_off.push_back(tile_off.back() + prep_tiles(problems[i]->prm.nx, problems[i]->prm.ny));
             if (problems[i]->prm.moving_boundary && !problems[i]->prm.periodic)
                 b->moving_nodes = std::max(b->moving_nodes, std::max(problems[i]->prm.nx, problems[i]->prm.ny));
         }
         b->total_blocks = blk_off.back();
+        b->total_tiles = tile_off.back();
         e = cudaMemcpy(b->blk_off_dev, blk_off.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(b->tile_off_dev, tile_off.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice);
         // the problem switches, when every problem shares them (the path kernel then has them compiled in)
         for (int i = 0; i < n; ++i) {
             const sdd_params& q = problems[i]->prm;

@@ -439,6 +439,11 @@ template <typename TI> __device__ __forceinline__ float chip_face(const void* f,
     if constexpr (sizeof(TI) == 8) return (float)f64[id];
     else return static_cast<const float*>(f)[id];
 }
+template <typename TI> __device__ __forceinline__ TI to_inner(double v)
+{
+    if constexpr (sizeof(TI) == 8) return v;
+    else return float_rn(v);
+}
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
@@ -777,11 +782,11 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
                 const double ay = fma_rn(-cS, P.ynew[id - nx], fma_rn(-cN, P.ynew[id + nx], fma_rn(-cW, P.ynew[id - 1],
                                   fma_rn(diag, P.ynew[id], -(cE * P.ynew[id + 1])))));
                 if (P.form == 0) {
-                    r[s].x = (TI)(P.xcur[id] - ax);
-                    r[s].y = (TI)(P.ycur[id] - ay);
+                    r[s].x = to_inner<TI>(P.xcur[id] - ax);
+                    r[s].y = to_inner<TI>(P.ycur[id] - ay);
                 } else {
-                    r[s].x = (TI)fma_rn(P.om64[id], P.xcur[id], -ax);
-                    r[s].y = (TI)fma_rn(P.om64[id], P.ycur[id], -ay);
+                    r[s].x = to_inner<TI>(fma_rn(P.om64[id], P.xcur[id], -ax));
+                    r[s].y = to_inner<TI>(fma_rn(P.om64[id], P.ycur[id], -ay));
                 }
                 mac(rr[0], r[s].x, r[s].x);
                 mac(rr[1], r[s].y, r[s].y);

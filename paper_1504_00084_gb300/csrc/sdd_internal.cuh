@@ -95,6 +95,24 @@ __device__ __forceinline__ double uniform_open(uint32_t w, double)
     return __hiloint2double((int)(0x3FF00000u | (w >> 12)), (int)(w << 20)) - 0x1.ffffffffp-1;
 }
 
+// (float)d, rounded to nearest even, by integer operations where d and the result are normal numbers or
+// zero: the conversion instruction waits for the FP64 unit (16 clocks a warp and SM).
+__device__ __forceinline__ float float_rn(double d)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    if ((hi << 1 | lo) == 0) return __uint_as_float(hi);
+    if (((hi >> 20) & 0x7FFu) - 0x381u > 0xFCu) return (float)d;
+    const uint64_t u = (((uint64_t)hi << 32) | lo) + 0x0FFFFFFFu + ((lo >> 29) & 1u);
+    return __uint_as_float(((uint32_t)(u >> 29) + 0x40000000u) | (hi & 0x80000000u));
+}
+__device__ __forceinline__ bool finite_bits(double d) { return (~__double2hiint(d) & 0x7FF00000) != 0; }
+// d > 0 (and not a NaN)
+__device__ __forceinline__ bool positive_bits(double d)
+{
+    const int hi = __double2hiint(d), lo = __double2loint(d);
+    return hi >= 0 && (hi | lo) != 0 && (hi < 0x7FF00000 || (hi == 0x7FF00000 && lo == 0));
+}
+
 // ---------------------------------------------------------------------------------------
 // Packed per-node data read by the path kernel.
 // ---------------------------------------------------------------------------------------
@@ -269,11 +287,15 @@ struct ReduceParams {
 struct PrepParams {
     int nx, ny, periodic, kind, n_params, precision;
     double Lx, Ly, t;
+    double gx, gy;             // (nx - 1) / 2, (ny - 1) / 2 (set_prep_consts)
     const double* t_dev;       // if set, the time is read from device memory (graph replays)
     const double* x;           // current mesh
     const double* y;
     const double* omega_in;    // nodal monitor (kind == NODAL)
     double params[64];
+    // bumps (set_prep_consts): w^2, 1 / w^2, and the squared distance beyond which the term leaves the sum
+    // unchanged
+    double bump_w2[16], bump_inv[16], bump_reach[16];
     double* om64;              // out: omega at the nodes (FP64)
     double* wxi64;             // out: FD gradient (FP64)
     double* weta64;
@@ -287,6 +309,11 @@ struct PrepParams {
     void* bnd;                 // out: the same in the path precision
     double* bnd_scratch;       // 2 (2 nx + 2 ny) doubles
 };
+
+// What a thread would otherwise work out for its one node: gx, gy, and for bumps (kind 3) w^2, its
+// reciprocal and the reach.  With amplitudes >= 0 the sum is at least 1, and a term below 2^-54 leaves it
+// unchanged: a e^-z < 2^-54 for z > (55 + exponent of a) ln 2.  A term is never skipped otherwise.
+void set_prep_consts(PrepParams& P);
 
 // Per-problem record of a batch step's batched launches (monitor and packing, moving boundary,
 // estimator shifts, Dirichlet scatter, copy of the new mesh).
@@ -303,6 +330,7 @@ struct SolveParams {
     int scheme;                // 0 backward Euler, 1 forward Euler substeps
     int fe_max_substeps;
     double r;                  // dt / tau
+    double hx, hy;             // 1 / (2 h^2) along xi, eta (set_face_consts)
     double rtol;
     int max_iter;
     const double* om64;        // omega at the nodes
@@ -322,6 +350,12 @@ struct SolveParams {
     int32_t* stat_ok;
     double* stat_res;          // per subdomain: final relative residual (max of x, y)
 };
+
+inline void set_face_consts(SolveParams& P)
+{
+    P.hx = 0.5 * ((double)(P.nx - 1) * (double)(P.nx - 1));
+    P.hy = 0.5 * ((double)(P.ny - 1) * (double)(P.ny - 1));
+}
 
 // Subdomain lines of an n-node direction split into P parts: part I spans nodes
 // split_line(I) .. split_line(I + 1) (equal parts when P divides n - 1).
@@ -436,8 +470,10 @@ cudaError_t launch_faces(const SolveParams& P, bool fp64_inner, cudaStream_t s);
 // entries, blocks of 256 threads as batch_blocks gives them; node work over the concatenated nodes).
 int batch_blocks(long n_nodes);
 // moving_nodes: the longest side of the problems with a moving boundary (0: none)
-cudaError_t launch_prep_batch(const BatchRec* R, const int32_t* blk_off, int n, int total_blocks, bool fp64,
-                              int moving_nodes, cudaStream_t s);
+// tile_off, total_tiles: as blk_off, of prep_tiles
+int prep_tiles(int nx, int ny);
+cudaError_t launch_prep_batch(const BatchRec* R, const int32_t* blk_off, const int32_t* tile_off, int n, int total_blocks,
+                              int total_tiles, bool fp64, int moving_nodes, cudaStream_t s);
 cudaError_t launch_shift_batch(const BatchRec* R, const int32_t* node_prob, int M, double* shift, cudaStream_t s);
 cudaError_t launch_scatter_batch(const BatchRec* R, const int32_t* blk_off, int n, int total_blocks,
                                  const int32_t* node_prob, int M, const double* est, cudaStream_t s);

