@@ -242,13 +242,19 @@ sdd_status run_prep(sdd_problem* p)
     P.mon = p->mon; P.disp = p->disp; P.bad = p->bad;
     P.moving_boundary = p->prm.moving_boundary; P.form = p->prm.form; P.r = p->prm.dt / p->prm.tau;
     P.bnd64 = p->bnd64; P.bnd = p->bnd; P.bnd_scratch = p->bnd_scratch;
-    SDD_CK(cudaMemsetAsync(p->bad, 0, 4, p->stream));
     SDD_CK(launch_prep(P, p->stream));
     p->launches += 2;
-    if (p->M > 0) {
-        SDD_CK(launch_shift(p->nodes, p->M, p->prm.nx, p->x, p->y, p->shift, p->stream));
-        p->launches += 1;
-    }
+    return SDD_OK;
+}
+
+// Node sums cleared, shifts and path totals set, for the nodes [lo, hi).
+sdd_status init_mc(sdd_problem* p, int lo, int hi)
+{
+    const int64_t n0 = p->prm.paths_per_node;
+    SDD_CK(launch_mc_init(p->M, n0, p->prm.se_target > 0 ? p->prm.max_paths_per_node : n0, p->acc, p->n_done, p->steps,
+                          p->paths_run, p->next_total, p->stream, p->n_interp > 0 ? p->iface_role : nullptr, lo, hi,
+                          NodeShifts{p->nodes, p->prm.nx, p->x, p->y, p->shift}));
+    p->launches += 1;
     return SDD_OK;
 }
 
@@ -321,9 +327,7 @@ sdd_status run_mc(sdd_problem* p, int lo = 0, int hi = -1)
     const int64_t n0 = p->prm.paths_per_node;
     const int64_t maxp = adaptive ? p->prm.max_paths_per_node : n0;
     if (hi < 0) hi = M;
-    SDD_CK(launch_mc_init(M, n0, maxp, p->acc, p->n_done, p->steps, p->paths_run, p->next_total, p->stream,
-                          p->n_interp > 0 ? p->iface_role : nullptr, lo, hi));
-    p->launches += 1;
+    SDD_TRY(init_mc(p, lo, hi));
     int n_timed = 0;
     PlanParams PP{};
     PP.M = M; PP.n_done = p->n_done; PP.next_total = p->next_total; PP.node_of = p->node_of;
@@ -342,6 +346,7 @@ sdd_status run_mc(sdd_problem* p, int lo = 0, int hi = -1)
         // fixed N: the number of launches is known, no host round trip
         const int64_t chunk = (int64_t)kTasksPerRound * p->task_paths;
         const int64_t rounds = (n0 + chunk - 1) / chunk;
+        RP.est = p->est; RP.se = p->se;
         for (int64_t r = 0; r < rounds; ++r) {
             SDD_CK(launch_plan(PP, p->stream));
             SDD_TRY(timed_mc_round(p, n_timed++));
@@ -373,8 +378,10 @@ sdd_status run_mc(sdd_problem* p, int lo = 0, int hi = -1)
             p->stats.mc_rounds = r + 1;
         }
     }
-    SDD_CK(launch_output(M, p->acc, p->n_done, p->shift, p->est, p->se, p->stream));
-    p->launches += 1;
+    if (adaptive) {
+        SDD_CK(launch_output(M, p->acc, p->n_done, p->shift, p->est, p->se, p->stream));
+        p->launches += 1;
+    }
     if (p->n_interp > 0) {
         SDD_CK(launch_interp(p->interp, p->n_interp, p->est, p->se, p->stream));
         p->launches += 1;
@@ -410,9 +417,6 @@ sdd_status run_mc(sdd_problem* p, int lo = 0, int hi = -1)
 sdd_status run_solve(sdd_problem* p)
 {
     const TraceRange trace("sdd: subdomain solves");
-    SDD_CK(launch_scatter(p->prm.nx, p->prm.ny, p->prm.periodic, p->prm.Lx, p->prm.Ly, p->nodes, p->M,
-                          p->est, p->xn, p->yn, p->stream, p->prm.moving_boundary ? p->bnd64 : nullptr));
-    p->launches += (p->prm.periodic ? 0 : 1) + (p->M > 0 ? 1 : 0);
     SolveParams S{};
     S.nx = p->prm.nx; S.ny = p->prm.ny; S.px = p->prm.px; S.py = p->prm.py; S.form = p->prm.form;
     S.r = p->prm.dt / p->prm.tau; set_face_consts(S); S.rtol = p->prm.solve_rtol; S.max_iter = p->prm.solve_max_iter;
@@ -426,6 +430,8 @@ sdd_status run_solve(sdd_problem* p)
     if (!p->solve_ev[0]) SDD_CK(cudaEventCreate(&p->solve_ev[0]));
     if (!p->solve_ev[1]) SDD_CK(cudaEventCreate(&p->solve_ev[1]));
     SDD_CK(cudaEventRecord(p->solve_ev[0], p->stream));
+    SDD_CK(launch_solve_setup(S, p->prm.periodic, p->prm.Lx, p->prm.Ly, p->nodes, p->M, p->est,
+                              p->prm.moving_boundary ? p->bnd64 : nullptr, p->fp64, p->stream));
     SDD_CK(launch_solve(S, p->plan, p->chip_items, p->solve_items, p->fp64, p->stream));
     SDD_CK(cudaEventRecord(p->solve_ev[1], p->stream));
     p->launches += 1 + (int)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1);
@@ -986,10 +992,7 @@ sdd_status sdd_tune(sdd_problem* p, int32_t tune_paths_per_task, sdd_mc_config* 
     if (p->M > 0) {
         SDD_TRY(run_prep(p));
         const int64_t n0 = p->prm.paths_per_node;
-        const int64_t maxp = p->prm.se_target > 0 ? p->prm.max_paths_per_node : n0;
-        SDD_CK(launch_mc_init(p->M, n0, maxp, p->acc, p->n_done, p->steps, p->paths_run, p->next_total,
-                              p->stream, p->n_interp > 0 ? p->iface_role : nullptr));
-        p->launches += 1;
+        SDD_TRY(init_mc(p, 0, p->M));
         PlanParams PP{};
         PP.M = p->M; PP.n_done = p->n_done; PP.next_total = p->next_total; PP.node_of = p->node_of;
         PP.p_begin = p->p_begin; PP.p_count = p->p_count; PP.task_off = p->task_off;
@@ -1164,6 +1167,8 @@ sdd_status sdd_debug_paths(sdd_problem* p, int32_t node, int64_t p_begin, int64_
     const int64_t tasks = (n_paths + p->task_paths - 1) / p->task_paths;
     if (tasks > p->slot_cap) return fail(SDD_ERR_INVALID_ARG, "too many paths for one debug call");
     SDD_TRY(run_prep(p));
+    SDD_CK(launch_shift(p->nodes, p->M, p->prm.nx, p->x, p->y, p->shift, p->stream));
+    p->launches += 1;
     double* dval = nullptr;
     int32_t* dst = nullptr;
     int8_t* dsd = nullptr;

@@ -282,6 +282,7 @@ struct ReduceParams {
     int64_t* next_total;
     double se_target;          // 0: fixed N
     int64_t max_paths;
+    double *est, *se;          // if set, the active nodes' estimates and standard errors so far
 };
 
 struct PrepParams {
@@ -442,15 +443,22 @@ cudaError_t launch_quality(int nx, int ny, const double* x, const double* y, dou
                            cudaStream_t s);
 cudaError_t launch_shift(const int2* nodes, int M, int nx, const double* x, const double* y,
                          double* shift, cudaStream_t s);
-// bnd64 (nullable): the moving boundary's new tangential coordinates (PrepParams layout)
-cudaError_t launch_scatter(int nx, int ny, int periodic, double Lx, double Ly, const int2* nodes,
-                           int M, const double* est, double* xnew, double* ynew, cudaStream_t s,
-                           const double* bnd64 = nullptr);
+// Rims of the new mesh (Dirichlet boundary; interface estimates) and the face coefficients, which
+// launch_solve needs.  bnd64 (nullable): the moving boundary's new tangential coordinates (PrepParams layout)
+cudaError_t launch_solve_setup(const SolveParams& P, int periodic, double Lx, double Ly, const int2* nodes, int M,
+                               const double* est, const double* bnd64, bool fp64_inner, cudaStream_t s);
+// The estimator shifts of M nodes (their current mesh points), written by launch_mc_init.
+struct NodeShifts {
+    const int2* nodes;
+    int nx;
+    const double *x, *y;
+    double* shift;
+};
 // role (nullable): per node, -1 = estimated by Monte Carlo, >= 0 = interpolated (never planned)
 // Nodes outside [lo, hi) (hi < 0: M) and interpolated nodes (role >= 0) are scheduled no paths.
 cudaError_t launch_mc_init(int M, int64_t n0, int64_t max_paths, double* acc, int64_t* n_done,
                            int64_t* steps, int64_t* paths_run, int64_t* next_total, cudaStream_t s,
-                           const int32_t* role = nullptr, int lo = 0, int hi = -1);
+                           const int32_t* role = nullptr, int lo = 0, int hi = -1, const NodeShifts& shifts = {});
 cudaError_t launch_interp(const InterpRule* rules, int n, double* est, double* se, cudaStream_t s);
 cudaError_t launch_plan(const PlanParams& P, cudaStream_t s);
 template <typename T>
@@ -462,10 +470,9 @@ template <typename T> int mc_max_blocks_per_sm(int acc_mode, bool debug, bool ba
 cudaError_t launch_reduce(const ReduceParams& P, int M, cudaStream_t s);
 cudaError_t launch_output(int M, const double* acc, const int64_t* n_done, const double* shift,
                           double* est, double* se, cudaStream_t s);
-// Face coefficients and subdomain solves of one problem (plan's items in device memory).
+// Subdomain solves of one problem (plan's items in device memory), after launch_solve_setup.
 cudaError_t launch_solve(const SolveParams& P, const SolvePlan& plan, const int2* chip_items, const SolveItem* items,
                          bool fp64_inner, cudaStream_t s);
-cudaError_t launch_faces(const SolveParams& P, bool fp64_inner, cudaStream_t s);
 // Batched launches of a batch step (blk_off: per-problem block offsets of grid-sized work, n + 1
 // entries, blocks of 256 threads as batch_blocks gives them; node work over the concatenated nodes).
 int batch_blocks(long n_nodes);

@@ -185,7 +185,7 @@ bool on_device(const void* p)
 
 template <typename T>
 sdd_status run(const sdd_params* P, const Buffers& b, int M, int acc_mode, int task_paths, int32_t step_index,
-               cudaStream_t s)
+               const NodeShifts& shifts, double* est, double* se, cudaStream_t s)
 {
     int dev = 0, nsm = 1;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -224,11 +224,12 @@ sdd_status run(const sdd_params* P, const Buffers& b, int M, int acc_mode, int t
     rp.slots = b.slots; rp.shift = b.shift; rp.acc = b.acc; rp.n_done = b.n_done; rp.steps = b.steps;
     rp.paths_run = b.paths_run; rp.next_total = b.next_total; rp.se_target = 0.0;
     rp.max_paths = P->paths_per_node;
+    rp.est = est; rp.se = se;
 
     const int grid = nsm * mc_max_blocks_per_sm<T>(acc_mode, false, false);
     const int64_t rounds = (P->paths_per_node + kMaxChunk - 1) / kMaxChunk;
     if (launch_mc_init(M, P->paths_per_node, P->paths_per_node, b.acc, b.n_done, b.steps, b.paths_run,
-                       b.next_total, s) != cudaSuccess)
+                       b.next_total, s, nullptr, 0, -1, shifts) != cudaSuccess)
         return SDD_ERR_CUDA;
     for (int64_t r = 0; r < rounds; ++r) {
         if (launch_plan(pp, s) != cudaSuccess) return SDD_ERR_CUDA;
@@ -295,13 +296,11 @@ extern "C" sdd_status sdd_interface_mc_noalloc(const sdd_params* P, const double
     pr.nx = P->nx; pr.ny = P->ny; pr.periodic = P->periodic; pr.kind = SDD_MONITOR_NODAL; pr.n_params = 0;
     pr.precision = P->precision; pr.Lx = P->Lx; pr.Ly = P->Ly; pr.t = P->t0 + step_index * P->dt;
     pr.x = x; pr.y = y; pr.omega_in = omega;
-    pr.om64 = b.om64; pr.wxi64 = b.wxi64; pr.weta64 = b.weta64; pr.mon = b.mon; pr.disp = b.disp;
+    pr.om64 = P->periodic ? b.om64 : const_cast<double*>(omega);  // read where it is unless it is to be wrapped
+    pr.wxi64 = b.wxi64; pr.weta64 = b.weta64; pr.mon = b.mon; pr.disp = b.disp;
     set_prep_consts(pr);
     if (launch_prep(pr, s) != cudaSuccess) return SDD_ERR_CUDA;
-    if (launch_shift(b.nodes, (int)M, P->nx, x, y, b.shift, s) != cudaSuccess) return SDD_ERR_CUDA;
-    const sdd_status r = fp64 ? run<double>(P, b, (int)M, acc_mode, task_paths, step_index, s)
-                              : run<float>(P, b, (int)M, acc_mode, task_paths, step_index, s);
-    if (r != SDD_OK) return r;
-    if (launch_output((int)M, b.acc, b.n_done, b.shift, est_xy, se_xy, s) != cudaSuccess) return SDD_ERR_CUDA;
-    return SDD_OK;
+    const NodeShifts shifts{b.nodes, P->nx, x, y, b.shift};
+    return fp64 ? run<double>(P, b, (int)M, acc_mode, task_paths, step_index, shifts, est_xy, se_xy, s)
+                : run<float>(P, b, (int)M, acc_mode, task_paths, step_index, shifts, est_xy, se_xy, s);
 }

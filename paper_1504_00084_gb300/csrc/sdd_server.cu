@@ -347,12 +347,10 @@ sdd_status admit(sdd_server* s, Request* r)
     P.bad = s->slot_bad + r->slot;
     P.moving_boundary = r->prm.moving_boundary; P.form = r->prm.form; P.r = r->prm.dt / r->prm.tau;
     P.bnd64 = p->bnd64; P.bnd = p->bnd; P.bnd_scratch = p->bnd_scratch;
-    S_CK(cudaMemsetAsync(P.bad, 0, 4, s->stream));
     S_CK(launch_prep(P, s->stream));
     s->st.kernel_launches += 2;
     if (r->M > 0) {
         const int64_t o = r->off;
-        S_CK(launch_shift(p->nodes, r->M, r->prm.nx, p->x, p->y, s->shift + 2 * o, s->stream));
         fill_i32_kernel<<<(r->M + 255) / 256, 256, 0, s->stream>>>(s->node_prob + o, r->M, r->slot);
         fill_i32_kernel<<<(r->M + 255) / 256, 256, 0, s->stream>>>(s->node_fill + o, r->M, p->fill());
         S_CK(cudaGetLastError());
@@ -360,8 +358,9 @@ sdd_status admit(sdd_server* s, Request* r)
         const int64_t n0 = s->prm.paths_per_node;
         const int64_t maxp = adaptive ? s->prm.max_paths_per_node : n0;
         S_CK(launch_mc_init(r->M, n0, maxp, s->acc + 4 * o, s->n_done + o, s->steps + o, s->paths_run + o,
-                            s->next_total + o, s->stream, p->n_interp > 0 ? p->iface_role : nullptr));
-        s->st.kernel_launches += 4;
+                            s->next_total + o, s->stream, p->n_interp > 0 ? p->iface_role : nullptr, 0, -1,
+                            NodeShifts{p->nodes, r->prm.nx, p->x, p->y, s->shift + 2 * o}));
+        s->st.kernel_launches += 3;
     }
     if (s->fp64) write_record<double>(s, r); else write_record<float>(s, r);
     const size_t rec = s->fp64 ? sizeof(McProblem<double>) : sizeof(McProblem<float>);
@@ -386,9 +385,6 @@ sdd_status finish(sdd_server* s, Request* r)
         S_CK(launch_interp(p->interp, p->n_interp, s->est + 2 * o, s->se + 2 * o, s->fin));
         s->st.kernel_launches += 1 + (p->n_interp > 0 ? 1 : 0);
     }
-    S_CK(launch_scatter(r->prm.nx, r->prm.ny, r->prm.periodic, r->prm.Lx, r->prm.Ly, p->nodes, r->M,
-                        s->est + 2 * o, p->xn, p->yn, s->fin, r->prm.moving_boundary ? p->bnd64 : nullptr));
-    s->st.kernel_launches += (r->prm.periodic ? 0 : 1) + (r->M > 0 ? 1 : 0);
     SolveParams S{};
     S.nx = r->prm.nx; S.ny = r->prm.ny; S.px = r->prm.px; S.py = r->prm.py; S.form = r->prm.form;
     S.r = r->prm.dt / r->prm.tau; set_face_consts(S); S.rtol = r->prm.solve_rtol; S.max_iter = r->prm.solve_max_iter;
@@ -398,6 +394,8 @@ sdd_status finish(sdd_server* s, Request* r)
     S.ce64 = p->ce64; S.cn64 = p->cn64; S.ce = p->ce; S.cn = p->cn; S.vec = p->vec;
     S.mg = p->mg; S.mg_stride = p->mg_stride;
     S.stat_iters = p->st_iters; S.stat_outer = p->st_outer; S.stat_ok = p->st_ok; S.stat_res = p->st_res;
+    S_CK(launch_solve_setup(S, r->prm.periodic, r->prm.Lx, r->prm.Ly, p->nodes, r->M, s->est + 2 * o,
+                            r->prm.moving_boundary ? p->bnd64 : nullptr, s->fp64, s->fin));
     S_CK(launch_solve(S, p->plan, p->chip_items, p->solve_items, s->fp64, s->fin));
     s->st.kernel_launches += 1 + (int64_t)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1);
     S_CK(cudaEventRecord(r->done_ev, s->fin));

@@ -154,44 +154,6 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh)
     __syncthreads();
 }
 
-__device__ __forceinline__ void faces_body(const SolveParams& P, int inner_fp64, int blk, int nb)
-{
-    const int nx = P.nx, ny = P.ny;
-    const long n = (long)nx * ny;
-    // r (w + w')/2 / h^2, each step rounded; the half is taken into 1 / h^2, which is exact.  4097 x 4097
-    // nodes: 0.45 -> 0.26 ms (44 bytes a node take 0.11) with fewer FP64 operations and conversions
-    for (int id = blk * (int)blockDim.x + threadIdx.x; id < n; id += nb * (int)blockDim.x) {  // n <= 2^28
-        const int j = id / nx, i = id - j * nx;
-        const double w = P.om64[id];
-        double e = 0.0, no = 0.0;
-        if (i < nx - 1) e = __dmul_rn(P.r, __dmul_rn(__dadd_rn(w, P.om64[id + 1]), P.hx));
-        if (j < ny - 1) no = __dmul_rn(P.r, __dmul_rn(__dadd_rn(w, P.om64[id + nx]), P.hy));
-        P.ce64[id] = e;
-        P.cn64[id] = no;
-        if (inner_fp64) {
-            static_cast<double*>(P.ce)[id] = e;
-            static_cast<double*>(P.cn)[id] = no;
-        } else {
-            static_cast<float*>(P.ce)[id] = float_rn(e);
-            static_cast<float*>(P.cn)[id] = float_rn(no);
-        }
-    }
-}
-
-__global__ void faces_kernel(const SolveParams P, int inner_fp64) { faces_body(P, inner_fp64, blockIdx.x, gridDim.x); }
-
-// Face coefficients of every problem of a batch in one launch (problem i: blocks blk_off[i] ..).
-__global__ void faces_batch_kernel(const SolveParams* probs, const int32_t* blk_off, int n, int inner_fp64)
-{
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (blk_off[mid] <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
-    }
-    faces_body(probs[lo], inner_fp64, blockIdx.x - blk_off[lo], blk_off[lo + 1] - blk_off[lo]);
-}
-
-
 // ------------------------------------------------------------------------------------------
 // Multigrid hierarchy of one subdomain: compact per-level arrays in the subdomain's workspace.
 // ------------------------------------------------------------------------------------------
@@ -970,20 +932,6 @@ cudaError_t launch_plan_solves(const SolveParams& P, const SolveParams* probs, c
 
 }  // namespace
 
-cudaError_t launch_faces_batch(const SolveParams* probs, const int32_t* blk_off, int n, int total_blocks,
-                               bool fp64_inner, cudaStream_t s)
-{
-    faces_batch_kernel<<<total_blocks, 256, 0, s>>>(probs, blk_off, n, fp64_inner ? 1 : 0);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_faces(const SolveParams& P, bool fp64_inner, cudaStream_t s)
-{
-    const long n = (long)P.nx * P.ny;
-    faces_kernel<<<(int)((n + 255) / 256), 256, 0, s>>>(P, fp64_inner ? 1 : 0);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const int2* chip_items,
                                const SolveItem* items, bool fp64_inner, cudaStream_t s)
 {
@@ -993,8 +941,7 @@ cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, 
 cudaError_t launch_solve(const SolveParams& P, const SolvePlan& plan, const int2* chip_items, const SolveItem* items,
                          bool fp64_inner, cudaStream_t s)
 {
-    const cudaError_t e = launch_faces(P, fp64_inner, s);
-    return e != cudaSuccess ? e : launch_plan_solves(P, nullptr, plan, chip_items, items, fp64_inner, s);
+    return launch_plan_solves(P, nullptr, plan, chip_items, items, fp64_inner, s);
 }
 
 }  // namespace sdd
