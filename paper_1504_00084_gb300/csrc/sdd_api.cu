@@ -209,6 +209,36 @@ sdd_status copy_out(sdd_problem* p, void* dst, const void* src, size_t bytes)
     return SDD_OK;
 }
 
+// Outputs of a call, queued on the stream before the host waits for it: a small result is copied through
+// the pinned staging block and handed over by flush_out; a device or larger destination gets its copy there,
+// when the status is known.  (A copy to pageable memory waits on its own, about 10 us each.)
+void begin_out(sdd_problem* p)
+{
+    p->stage_used = 0;
+    p->staged.clear();
+    p->late.clear();
+}
+sdd_status stage_out(sdd_problem* p, void* dst, const void* src, size_t bytes)
+{
+    if (!dst || bytes == 0) return SDD_OK;
+    const size_t at = (p->stage_used + 15) / 16 * 16;
+    if (at + bytes > p->stage_cap || is_device_ptr(dst)) {
+        p->late.push_back({dst, src, bytes});
+        return SDD_OK;
+    }
+    SDD_CK(cudaMemcpyAsync(p->h_stage + at, src, bytes, cudaMemcpyDeviceToHost, p->stream));
+    p->staged.push_back({dst, p->h_stage + at, bytes});
+    p->stage_used = at + bytes;
+    return SDD_OK;
+}
+sdd_status flush_out(sdd_problem* p)
+{
+    for (const sdd_problem::Out& o : p->staged) memcpy(o.dst, o.from, o.bytes);
+    for (const sdd_problem::Out& o : p->late) SDD_TRY(copy_out(p, o.dst, o.from, o.bytes));
+    begin_out(p);
+    return SDD_OK;
+}
+
 sdd_status check_boundary(const sdd_problem* p, const double* x, const double* y)
 {
     if (p->prm.periodic) return SDD_OK;
@@ -253,7 +283,7 @@ sdd_status init_mc(sdd_problem* p, int lo, int hi)
     const int64_t n0 = p->prm.paths_per_node;
     SDD_CK(launch_mc_init(p->M, n0, p->prm.se_target > 0 ? p->prm.max_paths_per_node : n0, p->acc, p->n_done, p->steps,
                           p->paths_run, p->next_total, p->stream, p->n_interp > 0 ? p->iface_role : nullptr, lo, hi,
-                          NodeShifts{p->nodes, p->prm.nx, p->x, p->y, p->shift}));
+                          McStart{p->nodes, p->prm.nx, p->x, p->y, p->shift, p->totals}));
     p->launches += 1;
     return SDD_OK;
 }
@@ -304,8 +334,8 @@ sdd_status timed_mc_round(sdd_problem* p, int slot)
 }
 
 // Interface Monte Carlo of the nodes [lo, hi) (hi < 0: all M); the other nodes take no paths and
-// their outputs are not meaningful.
-sdd_status run_mc(sdd_problem* p, int lo = 0, int hi = -1)
+// their outputs are not meaningful.  Queued: collect_mc reads its totals after the stream is synchronised.
+sdd_status queue_mc(sdd_problem* p, int lo = 0, int hi = -1)
 {
     const TraceRange trace("sdd: interface Monte Carlo");
     const int M = p->M;
@@ -316,11 +346,9 @@ sdd_status run_mc(sdd_problem* p, int lo = 0, int hi = -1)
     p->stats.paths = 0;
     p->stats.nodes_not_reached = 0;
     p->stats.max_se = 0.0;
+    p->mc_timed = 0;
     if (M == 0) {
         SDD_CK(cudaMemcpyAsync(p->h_n_active + 1, p->bad, 4, cudaMemcpyDeviceToHost, p->stream));
-        SDD_CK(cudaStreamSynchronize(p->stream));
-        if (p->h_n_active[1]) return fail(SDD_ERR_INVALID_ARG, "monitor must be finite and > 0, mesh finite");
-        p->have_est = true;
         return SDD_OK;
     }
     const bool adaptive = p->prm.se_target > 0;
@@ -386,35 +414,46 @@ sdd_status run_mc(sdd_problem* p, int lo = 0, int hi = -1)
         SDD_CK(launch_interp(p->interp, p->n_interp, p->est, p->se, p->stream));
         p->launches += 1;
     }
-    // counters (small copies)
-    std::vector<int64_t> st(M), np(M);
-    std::vector<double> se((size_t)2 * M);
-    SDD_CK(cudaMemcpyAsync(st.data(), p->steps, 8 * (size_t)M, cudaMemcpyDeviceToHost, p->stream));
-    SDD_CK(cudaMemcpyAsync(np.data(), p->paths_run, 8 * (size_t)M, cudaMemcpyDeviceToHost, p->stream));
-    SDD_CK(cudaMemcpyAsync(se.data(), p->se, 16 * (size_t)M, cudaMemcpyDeviceToHost, p->stream));
-    SDD_CK(cudaMemcpyAsync(p->h_n_active + 1, p->bad, 4, cudaMemcpyDeviceToHost, p->stream));
-    SDD_CK(cudaStreamSynchronize(p->stream));
-    if (p->h_n_active[1]) return fail(SDD_ERR_INVALID_ARG, "monitor must be finite and > 0, mesh finite");
-    p->stats.mc_kernel_ms = 0.0;
-    p->stats.mc_kernel_launches = n_timed;
-    for (int k = 0; k < n_timed; ++k) {
-        float ms = 0.f;
-        SDD_CK(cudaEventElapsedTime(&ms, p->ev[2 * k], p->ev[2 * k + 1]));
-        p->stats.mc_kernel_ms += ms;
-    }
-    for (int m = lo; m < hi; ++m) {
-        p->stats.path_steps += st[m];
-        p->stats.paths += np[m];
-        const double s = se[2 * m] > se[2 * m + 1] ? se[2 * m] : se[2 * m + 1];
-        if (s > p->stats.max_se) p->stats.max_se = s;
-        if (adaptive && s > p->prm.se_target) p->stats.nodes_not_reached += 1;
+    SDD_CK(launch_totals(lo, hi, p->steps, p->paths_run, p->se, adaptive ? p->prm.se_target : 0.0, p->bad, p->totals,
+                         p->stream));
+    p->launches += 1;
+    SDD_CK(cudaMemcpyAsync(p->h_totals, p->totals, sizeof(McTotals), cudaMemcpyDeviceToHost, p->stream));
+    p->mc_timed = n_timed;
+    return SDD_OK;
+}
+
+sdd_status collect_mc(sdd_problem* p)
+{
+    if (p->M > 0 ? p->h_totals->bad : p->h_n_active[1])
+        return fail(SDD_ERR_INVALID_ARG, "monitor must be finite and > 0, mesh finite");
+    if (p->M > 0) {
+        p->stats.mc_kernel_launches = p->mc_timed;
+        for (int k = 0; k < p->mc_timed; ++k) {
+            float ms = 0.f;
+            SDD_CK(cudaEventElapsedTime(&ms, p->ev[2 * k], p->ev[2 * k + 1]));
+            p->stats.mc_kernel_ms += ms;
+        }
+        p->stats.path_steps = (int64_t)p->h_totals->steps;
+        p->stats.paths = (int64_t)p->h_totals->paths;
+        memcpy(&p->stats.max_se, &p->h_totals->max_se, 8);
+        p->stats.nodes_not_reached = p->h_totals->not_reached;
     }
     p->have_est = true;
     return p->stats.nodes_not_reached ? fail(SDD_ERR_SE_NOT_REACHED, "max_paths_per_node reached before se_target")
                                       : SDD_OK;
 }
 
-sdd_status run_solve(sdd_problem* p)
+// Host copy of the solves' records.
+char* stat_place(sdd_problem* p)
+{
+    if (p->h_stats) return p->h_stats;
+    p->v_stats.resize((size_t)p->prm.px * p->prm.py * sdd_problem::kStatBytes);
+    return p->v_stats.data();
+}
+
+// Subdomain solves, queued; collect_solve reads their records after the stream is synchronised.  guarded:
+// they return at once if the preparation has found the monitor or the mesh invalid.
+sdd_status queue_solve(sdd_problem* p, bool guarded)
 {
     const TraceRange trace("sdd: subdomain solves");
     SolveParams S{};
@@ -426,6 +465,7 @@ sdd_status run_solve(sdd_problem* p)
     S.ce64 = p->ce64; S.cn64 = p->cn64; S.ce = p->ce; S.cn = p->cn; S.vec = p->vec;
     S.mg = p->mg; S.mg_stride = p->mg_stride;
     S.stat_iters = p->st_iters; S.stat_outer = p->st_outer; S.stat_ok = p->st_ok; S.stat_res = p->st_res;
+    S.bad = guarded ? p->bad : nullptr;
     // device time of the solve launches
     if (!p->solve_ev[0]) SDD_CK(cudaEventCreate(&p->solve_ev[0]));
     if (!p->solve_ev[1]) SDD_CK(cudaEventCreate(&p->solve_ev[1]));
@@ -435,14 +475,16 @@ sdd_status run_solve(sdd_problem* p)
     SDD_CK(launch_solve(S, p->plan, p->chip_items, p->solve_items, p->fp64, p->stream));
     SDD_CK(cudaEventRecord(p->solve_ev[1], p->stream));
     p->launches += 1 + (int)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1);
+    SDD_CK(cudaMemcpyAsync(stat_place(p), p->st_res, (size_t)p->prm.px * p->prm.py * sdd_problem::kStatBytes,
+                           cudaMemcpyDeviceToHost, p->stream));
+    return SDD_OK;
+}
+
+sdd_status collect_solve(sdd_problem* p)
+{
     const int ns = p->prm.px * p->prm.py;
-    std::vector<int32_t> it(ns), ou(ns), ok(ns);
-    std::vector<double> rs(ns);
-    SDD_CK(cudaMemcpyAsync(it.data(), p->st_iters, 4 * (size_t)ns, cudaMemcpyDeviceToHost, p->stream));
-    SDD_CK(cudaMemcpyAsync(ou.data(), p->st_outer, 4 * (size_t)ns, cudaMemcpyDeviceToHost, p->stream));
-    SDD_CK(cudaMemcpyAsync(ok.data(), p->st_ok, 4 * (size_t)ns, cudaMemcpyDeviceToHost, p->stream));
-    SDD_CK(cudaMemcpyAsync(rs.data(), p->st_res, 8 * (size_t)ns, cudaMemcpyDeviceToHost, p->stream));
-    SDD_CK(cudaStreamSynchronize(p->stream));
+    const double* rs = reinterpret_cast<const double*>(stat_place(p));
+    const int32_t *it = reinterpret_cast<const int32_t*>(rs + ns), *ou = it + ns, *ok = ou + ns;
     p->stats.solve_iters_max = 0;
     p->stats.solve_outer_max = 0;
     p->stats.solve_rel_residual = 0.0;
@@ -461,20 +503,51 @@ sdd_status run_solve(sdd_problem* p)
     return bad ? fail(SDD_ERR_NOT_CONVERGED, "a subdomain solve reached solve_max_iter") : SDD_OK;
 }
 
-// The new mesh becomes the current one; time and the step index advance.
-sdd_status advance(sdd_problem* p, double* x_out, double* y_out)
+// The new mesh becomes the current one.
+void swap_mesh(sdd_problem* p)
 {
-    double* t;
-    t = p->x; p->x = p->xn; p->xn = t;
-    t = p->y; p->y = p->yn; p->yn = t;
+    std::swap(p->x, p->xn);
+    std::swap(p->y, p->yn);
+}
+
+// Time and the step index advance.
+void advance(sdd_problem* p)
+{
+    swap_mesh(p);
     p->step += 1;
     p->have_est = false;
     p->stats.step_index = (int32_t)p->step;
     p->stats.t = p->prm.t0 + (double)p->step * p->prm.dt;
-    const size_t N = (size_t)p->prm.nx * p->prm.ny;
-    SDD_TRY(copy_out(p, x_out, p->x, N * 8));
-    SDD_TRY(copy_out(p, y_out, p->y, N * 8));
-    return SDD_OK;
+}
+
+// A step's Monte Carlo and solves, with x_out and y_out staged, and one wait.  The solves start before the
+// host knows the Monte Carlo's status; they are guarded, and a failed step leaves the state as it was.
+sdd_status step_work(sdd_problem* p, double* x_out, double* y_out, sdd_status* s_mc, sdd_status* s_sv)
+{
+    begin_out(p);
+    SDD_TRY(run_prep(p));
+    SDD_TRY(queue_mc(p));
+    SDD_TRY(queue_solve(p, true));
+    const size_t bytes = (size_t)p->prm.nx * p->prm.ny * 8;
+    SDD_TRY(stage_out(p, x_out, p->xn, bytes));
+    SDD_TRY(stage_out(p, y_out, p->yn, bytes));
+    SDD_CK(cudaStreamSynchronize(p->stream));
+    *s_mc = collect_mc(p);
+    if (*s_mc != SDD_OK && *s_mc != SDD_ERR_SE_NOT_REACHED) return *s_mc;
+    *s_sv = collect_solve(p);
+    return *s_sv != SDD_OK && *s_sv != SDD_ERR_NOT_CONVERGED ? *s_sv : SDD_OK;
+}
+
+// Solves of given or earlier estimates, with x_out and y_out staged.
+sdd_status solve_work(sdd_problem* p, double* x_out, double* y_out)
+{
+    SDD_TRY(queue_solve(p, false));
+    begin_out(p);
+    const size_t bytes = (size_t)p->prm.nx * p->prm.ny * 8;
+    SDD_TRY(stage_out(p, x_out, p->xn, bytes));
+    SDD_TRY(stage_out(p, y_out, p->yn, bytes));
+    SDD_CK(cudaStreamSynchronize(p->stream));
+    return collect_solve(p);
 }
 }  // namespace
 
@@ -508,11 +581,11 @@ void problem_arrays(sdd_problem* p, bool with_mc, F&& f)
         f((void**)&p->task_off, (M + 2) * 8); f((void**)&p->task_len, (M + 1) * 4); f((void**)&p->n_active, 16); f((void**)&p->task_counter, 16);
         f((void**)&p->slots, (size_t)p->slot_cap * sizeof(TaskSlot));
         f((void**)&p->est, (M + 1) * 16); f((void**)&p->se, (M + 1) * 16);
+        f((void**)&p->totals, sizeof(McTotals));
     }
     f((void**)&p->ce64, N * 8); f((void**)&p->cn64, N * 8); f((void**)&p->ce, N * rs); f((void**)&p->cn, N * rs);
     f((void**)&p->vec, N * 4 * 2 * rs);
-    f((void**)&p->st_iters, (size_t)ns * 4); f((void**)&p->st_outer, (size_t)ns * 4);
-    f((void**)&p->st_ok, (size_t)ns * 4); f((void**)&p->st_res, (size_t)ns * 8);
+    f((void**)&p->st_res, (size_t)ns * sdd_problem::kStatBytes);
     f((void**)&p->quality, (N + 2) * 8);
     f((void**)&p->mg, p->mg_stride * ns);
     f((void**)&p->bad, 16);
@@ -585,7 +658,23 @@ sdd_status sdd_alloc_problem(const sdd_params& prm, cudaStream_t stream, bool wi
         if (e == cudaSuccess) e = p->dalloc(ptr, b);
         if (e == cudaSuccess) p->dev_bytes += alloc_rounded(b);
     });
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&p->h_n_active, 32, cudaHostAllocDefault);
+    p->set_stat_places();
+    // the pinned block: counters, and (with Monte Carlo) the solves' records and the staging, as far as they
+    // are small: 512 KiB is a 180 x 180 mesh, which the copies take 10 us for; beyond, waiting for a copy to
+    // pageable memory costs little beside the copy
+    {
+        const size_t stats = (size_t)prm.px * prm.py * sdd_problem::kStatBytes;
+        const size_t mesh = (size_t)prm.nx * prm.ny * 16, nodes = (size_t)p->M * 40 + 32;
+        auto small = [](size_t b) { return b <= ((size_t)512 << 10) ? b : 0; };
+        const size_t n_stats = with_mc ? (small(stats) + 15) / 16 * 16 : 0;
+        p->stage_cap = with_mc ? std::max(small(mesh) + 16, small(nodes)) : 0;
+        char* h = nullptr;
+        if (e == cudaSuccess) e = cudaHostAlloc((void**)&h, 128 + n_stats + p->stage_cap, cudaHostAllocDefault);
+        p->h_n_active = reinterpret_cast<int32_t*>(h);
+        p->h_totals = reinterpret_cast<McTotals*>(h + 64);
+        if (n_stats) p->h_stats = h + 128;
+        p->h_stage = h + 128 + n_stats;
+    }
     for (int k = 0; k <= kRoundsAhead && e == cudaSuccess; ++k)
         e = cudaEventCreateWithFlags(&p->count_ev[k], cudaEventDisableTiming);
     if (e != cudaSuccess) {
@@ -807,12 +896,16 @@ sdd_status sdd_interface_mc(sdd_problem* p, double* est_xy, double* se_xy, int64
 {
     if (!p) return fail(SDD_ERR_INVALID_ARG, "problem is NULL");
     SDD_TRY(run_prep(p));
-    const sdd_status s = run_mc(p);
-    if (s != SDD_OK && s != SDD_ERR_SE_NOT_REACHED) return s;
+    SDD_TRY(queue_mc(p));
     const size_t M = (size_t)p->M;
-    SDD_TRY(copy_out(p, est_xy, p->est, M * 16));
-    SDD_TRY(copy_out(p, se_xy, p->se, M * 16));
-    SDD_TRY(copy_out(p, paths_used, p->n_done, M * 8));
+    begin_out(p);
+    SDD_TRY(stage_out(p, est_xy, p->est, M * 16));
+    SDD_TRY(stage_out(p, se_xy, p->se, M * 16));
+    SDD_TRY(stage_out(p, paths_used, p->n_done, M * 8));
+    SDD_CK(cudaStreamSynchronize(p->stream));
+    const sdd_status s = collect_mc(p);
+    if (s != SDD_OK && s != SDD_ERR_SE_NOT_REACHED) return s;
+    SDD_TRY(flush_out(p));
     return s;
 }
 
@@ -825,11 +918,9 @@ sdd_status sdd_subdomain_solve(sdd_problem* p, const double* iface_xy, double* x
         p->have_est = true;
     }
     if (!p->have_est) return fail(SDD_ERR_INVALID_ARG, "no interface data: pass iface_xy or call sdd_interface_mc");
-    const sdd_status s = run_solve(p);
+    const sdd_status s = solve_work(p, x_out, y_out);
     if (s != SDD_OK && s != SDD_ERR_NOT_CONVERGED) return s;
-    const size_t N = (size_t)p->prm.nx * p->prm.ny;
-    SDD_TRY(copy_out(p, x_out, p->xn, N * 8));
-    SDD_TRY(copy_out(p, y_out, p->yn, N * 8));
+    SDD_TRY(flush_out(p));
     return s;
 }
 
@@ -837,12 +928,10 @@ sdd_status sdd_step(sdd_problem* p, double* x_out, double* y_out)
 {
     if (!p) return fail(SDD_ERR_INVALID_ARG, "problem is NULL");
     const TraceRange trace("sdd_step");
-    SDD_TRY(run_prep(p));
-    const sdd_status s_mc = run_mc(p);
-    if (s_mc != SDD_OK && s_mc != SDD_ERR_SE_NOT_REACHED) return s_mc;
-    const sdd_status s_sv = run_solve(p);
-    if (s_sv != SDD_OK && s_sv != SDD_ERR_NOT_CONVERGED) return s_sv;
-    SDD_TRY(advance(p, x_out, y_out));
+    sdd_status s_mc = SDD_OK, s_sv = SDD_OK;
+    SDD_TRY(step_work(p, x_out, y_out, &s_mc, &s_sv));
+    advance(p);
+    SDD_TRY(flush_out(p));
     if (s_mc != SDD_OK) return fail(s_mc, "max_paths_per_node reached before se_target");
     return s_sv;
 }
@@ -857,12 +946,16 @@ sdd_status sdd_interface_mc_range(sdd_problem* p, int32_t node_begin, int32_t no
         return fail(SDD_ERR_INVALID_ARG, "interface sampling: interpolated nodes need the estimates of every range");
     SDD_TRY(run_prep(p));
     if (node_end == node_begin) return SDD_OK;
-    const sdd_status s = run_mc(p, node_begin, node_end);
-    if (s != SDD_OK && s != SDD_ERR_SE_NOT_REACHED) return s;
+    SDD_TRY(queue_mc(p, node_begin, node_end));
     const size_t b = (size_t)node_begin, n = (size_t)(node_end - node_begin);
-    SDD_TRY(copy_out(p, est_xy ? est_xy + 2 * b : nullptr, p->est + 2 * b, n * 16));
-    SDD_TRY(copy_out(p, se_xy ? se_xy + 2 * b : nullptr, p->se + 2 * b, n * 16));
-    SDD_TRY(copy_out(p, paths_used ? paths_used + b : nullptr, p->n_done + b, n * 8));
+    begin_out(p);
+    SDD_TRY(stage_out(p, est_xy ? est_xy + 2 * b : nullptr, p->est + 2 * b, n * 16));
+    SDD_TRY(stage_out(p, se_xy ? se_xy + 2 * b : nullptr, p->se + 2 * b, n * 16));
+    SDD_TRY(stage_out(p, paths_used ? paths_used + b : nullptr, p->n_done + b, n * 8));
+    SDD_CK(cudaStreamSynchronize(p->stream));
+    const sdd_status s = collect_mc(p);
+    if (s != SDD_OK && s != SDD_ERR_SE_NOT_REACHED) return s;
+    SDD_TRY(flush_out(p));
     p->have_est = false;  // the problem's own estimates cover this range only
     return s;
 }
@@ -873,9 +966,10 @@ sdd_status sdd_step_from_interface(sdd_problem* p, const double* iface_xy, doubl
     if (!iface_xy && p->M > 0) return fail(SDD_ERR_INVALID_ARG, "iface_xy is NULL");
     SDD_TRY(run_prep(p));
     if (p->M > 0) SDD_TRY(copy_in(p, p->est, iface_xy, (size_t)p->M * 16));
-    const sdd_status s_sv = run_solve(p);
+    const sdd_status s_sv = solve_work(p, x_out, y_out);
     if (s_sv != SDD_OK && s_sv != SDD_ERR_NOT_CONVERGED) return s_sv;
-    SDD_TRY(advance(p, x_out, y_out));
+    advance(p);
+    SDD_TRY(flush_out(p));
     return s_sv;
 }
 
@@ -895,16 +989,11 @@ sdd_status sdd_step_mkp(sdd_problem* p, int32_t K, double* x_out, double* y_out)
     int k = 0;
     for (; k < K; ++k) {
         p->step = n * K + k;
-        hard = run_prep(p);
+        sdd_status s_mc = SDD_OK, s_sv = SDD_OK;
+        hard = step_work(p, k == K - 1 ? x_out : nullptr, k == K - 1 ? y_out : nullptr, &s_mc, &s_sv);
         if (hard != SDD_OK) break;
-        const sdd_status s_mc = run_mc(p);
-        if (s_mc != SDD_OK && s_mc != SDD_ERR_SE_NOT_REACHED) { hard = s_mc; break; }
-        const sdd_status s_sv = run_solve(p);
-        if (s_sv != SDD_OK && s_sv != SDD_ERR_NOT_CONVERGED) { hard = s_sv; break; }
         if (soft == SDD_OK) soft = s_mc != SDD_OK ? s_mc : s_sv;
-        double* t;
-        t = p->x; p->x = p->xn; p->xn = t;
-        t = p->y; p->y = p->yn; p->yn = t;
+        swap_mesh(p);
         acc.path_steps += p->stats.path_steps;
         acc.paths += p->stats.paths;
         acc.mc_rounds += p->stats.mc_rounds;
@@ -938,9 +1027,7 @@ sdd_status sdd_step_mkp(sdd_problem* p, int32_t K, double* x_out, double* y_out)
     p->stats.solve_rel_residual = acc.solve_rel_residual;
     p->stats.step_index = (int32_t)p->step;
     p->stats.t = p->prm.t0 + (double)p->step * p->prm.dt;
-    const size_t N = (size_t)p->prm.nx * p->prm.ny;
-    SDD_TRY(copy_out(p, x_out, p->x, N * 8));
-    SDD_TRY(copy_out(p, y_out, p->y, N * 8));
+    SDD_TRY(flush_out(p));
     if (soft == SDD_ERR_SE_NOT_REACHED) return fail(soft, "max_paths_per_node reached before se_target");
     if (soft == SDD_ERR_NOT_CONVERGED) return fail(soft, "a subdomain solve reached solve_max_iter");
     return SDD_OK;

@@ -924,6 +924,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ So
     const int2 it = items[team];
     if (threadIdx.x == 0) sp = probs ? probs[it.x] : P;
     __syncthreads();
+    if (sp.bad && *sp.bad) return;  // alike in every CTA of a cluster
     chip_body<TI, CL, NS>(sp, it.y, L, &scal, chip_sm);
 }
 
@@ -1102,6 +1103,7 @@ __global__ void __launch_bounds__(kFeThreads, 1) fe_chip_kernel(const __grid_con
     const int2 it = items[team];
     if (threadIdx.x == 0) sp = probs ? probs[it.x] : P;
     __syncthreads();
+    if (sp.bad && *sp.bad) return;  // alike in every CTA of a cluster
     fe_chip_body<CL>(sp, it.y, chip_sm);
 }
 

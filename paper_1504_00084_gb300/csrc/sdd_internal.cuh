@@ -350,6 +350,7 @@ struct SolveParams {
     int32_t* stat_outer;
     int32_t* stat_ok;
     double* stat_res;          // per subdomain: final relative residual (max of x, y)
+    const int32_t* bad;        // if set and nonzero, the inputs are invalid: the solves return at once
 };
 
 inline void set_face_consts(SolveParams& P)
@@ -447,18 +448,28 @@ cudaError_t launch_shift(const int2* nodes, int M, int nx, const double* x, cons
 // launch_solve needs.  bnd64 (nullable): the moving boundary's new tangential coordinates (PrepParams layout)
 cudaError_t launch_solve_setup(const SolveParams& P, int periodic, double Lx, double Ly, const int2* nodes, int M,
                                const double* est, const double* bnd64, bool fp64_inner, cudaStream_t s);
-// The estimator shifts of M nodes (their current mesh points), written by launch_mc_init.
-struct NodeShifts {
+// What launch_mc_init sets beside the node sums: the estimator shifts of the nodes (their current mesh
+// points) and, to zero, the totals that launch_totals adds to.  Null: left as they are.
+struct McTotals {
+    unsigned long long steps, paths, max_se;  // max_se: the bits of a double >= 0
+    int32_t not_reached, bad;
+};
+struct McStart {
     const int2* nodes;
     int nx;
     const double *x, *y;
     double* shift;
+    McTotals* totals;
 };
+// Totals of the nodes [lo, hi): substeps, paths, the largest standard error and the nodes above se_target
+// (> 0), and the flag `bad`.
+cudaError_t launch_totals(int lo, int hi, const int64_t* steps, const int64_t* paths, const double* se, double se_target,
+                          const int32_t* bad, McTotals* out, cudaStream_t s);
 // role (nullable): per node, -1 = estimated by Monte Carlo, >= 0 = interpolated (never planned)
 // Nodes outside [lo, hi) (hi < 0: M) and interpolated nodes (role >= 0) are scheduled no paths.
 cudaError_t launch_mc_init(int M, int64_t n0, int64_t max_paths, double* acc, int64_t* n_done,
                            int64_t* steps, int64_t* paths_run, int64_t* next_total, cudaStream_t s,
-                           const int32_t* role = nullptr, int lo = 0, int hi = -1, const NodeShifts& shifts = {});
+                           const int32_t* role = nullptr, int lo = 0, int hi = -1, const McStart& start = {});
 cudaError_t launch_interp(const InterpRule* rules, int n, double* est, double* se, cudaStream_t s);
 cudaError_t launch_plan(const PlanParams& P, cudaStream_t s);
 template <typename T>

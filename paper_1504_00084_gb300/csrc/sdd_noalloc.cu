@@ -185,7 +185,7 @@ bool on_device(const void* p)
 
 template <typename T>
 sdd_status run(const sdd_params* P, const Buffers& b, int M, int acc_mode, int task_paths, int32_t step_index,
-               const NodeShifts& shifts, double* est, double* se, cudaStream_t s)
+               const McStart& shifts, double* est, double* se, cudaStream_t s)
 {
     int dev = 0, nsm = 1;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -300,7 +300,7 @@ extern "C" sdd_status sdd_interface_mc_noalloc(const sdd_params* P, const double
     pr.wxi64 = b.wxi64; pr.weta64 = b.weta64; pr.mon = b.mon; pr.disp = b.disp;
     set_prep_consts(pr);
     if (launch_prep(pr, s) != cudaSuccess) return SDD_ERR_CUDA;
-    const NodeShifts shifts{b.nodes, P->nx, x, y, b.shift};
+    const McStart shifts{b.nodes, P->nx, x, y, b.shift, nullptr};
     return fp64 ? run<double>(P, b, (int)M, acc_mode, task_paths, step_index, shifts, est_xy, se_xy, s)
                 : run<float>(P, b, (int)M, acc_mode, task_paths, step_index, shifts, est_xy, se_xy, s);
 }

@@ -76,15 +76,32 @@ struct sdd_problem {
     sdd::SolvePlan plan;            // how the subdomains are solved (backward Euler)
     sdd::SolveItem* solve_items = nullptr;
     int2* chip_items = nullptr;
+    double* st_res = nullptr;       // per subdomain; st_iters, st_outer and st_ok lie behind it (set_stat_places)
     int32_t *st_iters = nullptr, *st_outer = nullptr, *st_ok = nullptr;
-    double* st_res = nullptr;
+    static constexpr size_t kStatBytes = 20;  // of a subdomain
+    void set_stat_places()
+    {
+        const size_t ns = (size_t)prm.px * prm.py;
+        st_iters = reinterpret_cast<int32_t*>(st_res + ns);
+        st_outer = st_iters + ns;
+        st_ok = st_outer + ns;
+    }
     double* quality = nullptr;      // (nx-1)(ny-1) cell qualities + 2 stats
     int32_t* bad = nullptr;         // set by the monitor preparation on invalid monitor or mesh
     double* bnd64 = nullptr;        // moving boundary: new tangential boundary coordinates (FP64)
     void* bnd = nullptr;            //   the same in the path precision
     double* bnd_scratch = nullptr;  //   tridiagonal sweeps
-    // host
-    int32_t* h_n_active = nullptr;  // pinned: [0] active nodes, [1] invalid-input flag, [2..] round counts
+    sdd::McTotals* totals = nullptr;
+    // host: one pinned block.  [0] active nodes, [1] invalid-input flag, [2..] round counts; from byte 64 the
+    // totals; then the solves' records (if h_stats is set) and the staging of a step's outputs
+    int32_t* h_n_active = nullptr;
+    sdd::McTotals* h_totals = nullptr;
+    char *h_stats = nullptr, *h_stage = nullptr;
+    size_t stage_cap = 0, stage_used = 0;
+    struct Out { void* dst; const void* from; size_t bytes; };
+    std::vector<Out> staged, late;  // copies to the caller: from the staging, or made after the status is known
+    std::vector<char> v_stats;      // the solves' records when they have no pinned place
+    int mc_lo = 0, mc_hi = 0, mc_timed = 0;  // of the Monte Carlo that is queued
     cudaEvent_t count_ev[sdd::kRoundsAhead + 1] = {};  // after the copies of the round counts
     sdd_stats stats{};
     std::vector<void*> allocs;

@@ -359,7 +359,7 @@ sdd_status admit(sdd_server* s, Request* r)
         const int64_t maxp = adaptive ? s->prm.max_paths_per_node : n0;
         S_CK(launch_mc_init(r->M, n0, maxp, s->acc + 4 * o, s->n_done + o, s->steps + o, s->paths_run + o,
                             s->next_total + o, s->stream, p->n_interp > 0 ? p->iface_role : nullptr, 0, -1,
-                            NodeShifts{p->nodes, r->prm.nx, p->x, p->y, s->shift + 2 * o}));
+                            McStart{p->nodes, r->prm.nx, p->x, p->y, s->shift + 2 * o, nullptr}));
         s->st.kernel_launches += 3;
     }
     if (s->fp64) write_record<double>(s, r); else write_record<float>(s, r);

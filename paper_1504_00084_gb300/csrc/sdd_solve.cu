@@ -724,6 +724,7 @@ __global__ void __launch_bounds__(kSolveThreads) fe_kernel(const __grid_constant
     const int2 o = items[blockIdx.x];
     if (threadIdx.x == 0) sp = probs ? probs[o.x] : P;
     __syncthreads();
+    if (sp.bad && *sp.bad) return;
     fe_body(sp, o.y, sh);
 }
 
@@ -762,6 +763,7 @@ __global__ void __cluster_dims__(kCoopWidth, 1, 1) __launch_bounds__(kSolveThrea
     solve_items_kernel(const __grid_constant__ SolveParams P, const SolveItem* items)
 {
     __shared__ double sh[32 * 8 + 8];
+    if (P.bad && *P.bad) return;  // alike in every CTA of a cluster
     solve_item<TI>(P, items[blockIdx.x], sh);
 }
 
