@@ -83,6 +83,7 @@ struct sdd_batch {
     cudaGraphExec_t graph = nullptr;
     std::vector<const double*> graph_x;  // mesh pointers the graph was recorded with
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    SolveStreams solve_streams;
     cudaEvent_t sev0 = nullptr, sev1 = nullptr;  // around the batched face + solve launches
     cudaEvent_t count_ev[kRoundsAhead + 1] = {};  // after the round-count copies to h_n_active[2..]
     int64_t launches = 0;
@@ -123,6 +124,7 @@ struct sdd_batch {
         if (sev1) cudaEventDestroy(sev1);
         for (cudaEvent_t c : count_ev)
             if (c) cudaEventDestroy(c);
+        solve_streams.destroy();
         for (void* v : allocs) cudaFree(v);
         for (void* v : host_allocs) cudaFreeHost(v);
     }
@@ -322,7 +324,7 @@ sdd_status record_step(sdd_batch* b, bool first_plan = false)
     B_CK(launch_faces_batch(b->solve_dev, b->blk_off_dev, b->n, b->total_blocks, fp64_inner, b->stream));
     launches += 1;
     B_CK(cudaEventRecord(b->sev0, b->stream));
-    B_CK(launch_solve_batch(b->solve_dev, b->plan, b->chip_items_dev, b->items_dev, fp64_inner, b->stream));
+    B_CK(launch_solve_batch(b->solve_dev, b->plan, b->solve_streams, b->chip_items_dev, b->items_dev, fp64_inner, b->stream));
     B_CK(cudaEventRecord(b->sev1, b->stream));
     launches += (int64_t)b->plan.chip.size() + (b->plan.items.empty() ? 0 : 1);
     B_CK(launch_copy_back_batch(b->rec_dev, b->blk_off_dev, b->n, b->total_blocks, b->stream));
@@ -401,6 +403,7 @@ sdd_status sdd_batch_create(sdd_problem* const* problems, int32_t n, void* strea
     if (e == cudaSuccess) e = cudaEventCreate(&b->ev1);
     if (e == cudaSuccess) e = cudaEventCreate(&b->sev0);
     if (e == cudaSuccess) e = cudaEventCreate(&b->sev1);
+    if (e == cudaSuccess) e = b->solve_streams.create();
     for (int k = 0; k <= kRoundsAhead && e == cudaSuccess; ++k)
         e = cudaEventCreateWithFlags(&b->count_ev[k], cudaEventDisableTiming);
     if (e == cudaSuccess && b->M > 0)

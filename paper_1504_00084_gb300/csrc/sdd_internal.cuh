@@ -396,6 +396,17 @@ struct SolvePlan {
     std::vector<int2> chip_items;   // (problem, subdomain)
     std::vector<SolveItem> items;
 };
+// Side streams on which the classes of a plan run beside each other: a class leaves SMs idle in its last wave,
+// and clusters of 16 all the time (one fits on a GPC of 18 to 20 SMs).  They hang on the caller's stream by
+// events (also when it is captured).  Five classes of a batch of sixteen problems took 0.79, 0.62, 0.29, 0.17 and
+// 0.11 ms one after the other; beside each other the batch's step takes 0.9 ms less.
+struct SolveStreams {
+    static constexpr int kSide = 3;
+    cudaStream_t side[kSide] = {};
+    cudaEvent_t fork = nullptr, join[kSide] = {};
+    cudaError_t create();
+    void destroy();
+};
 // The plan of the subdomains of one problem's split (solve_subs), or of several problems'.
 SolvePlan solve_plan(std::vector<SolveSub> subs, bool fp64);
 // Subdomains of an nx x ny grid split px x py, appended to `subs` as problem `prob`.
@@ -499,7 +510,7 @@ cudaError_t launch_copy_back_batch(const BatchRec* R, const int32_t* blk_off, in
 cudaError_t launch_faces_batch(const SolveParams* probs, const int32_t* blk_off, int n, int total_blocks,
                                bool fp64_inner, cudaStream_t s);
 // Subdomain solves of a batch (plan's items in device memory).
-cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const int2* chip_items,
+cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const SolveStreams& side, const int2* chip_items,
                                const SolveItem* items, bool fp64_inner, cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, const uint32_t* key, int64_t n, uint32_t* out,
                           cudaStream_t s);

@@ -897,26 +897,40 @@ cudaError_t launch_chip_team(const SolveParams& P, const SolveParams* probs, con
                     : launch_chip_class(chip_kernel<TI, false, NS>, false, P, probs, c, items, s);
 }
 
-// The on-chip launches of a plan, then the global-memory one.
-cudaError_t launch_plan_solves(const SolveParams& P, const SolveParams* probs, const SolvePlan& plan,
-                               const int2* chip_items, const SolveItem* items, bool fp64_inner, cudaStream_t s)
+cudaError_t launch_chip(const SolveParams& P, const SolveParams* probs, const ChipLaunch& c, const int2* items,
+                        bool fp64_inner, cudaStream_t s)
 {
-    for (const ChipLaunch& c : plan.chip) {
-        cudaError_t e;
-        if (c.slots == 0) {
-            if (c.cw == 0) {
-                fe_kernel<<<c.count, kSolveThreads, 0, s>>>(P, probs, chip_items + c.first);
-                e = cudaGetLastError();
-            } else {
-                e = c.cw > 1 ? launch_chip_class(fe_chip_kernel<true>, true, P, probs, c, chip_items, s)
-                             : launch_chip_class(fe_chip_kernel<false>, false, P, probs, c, chip_items, s);
-            }
-        } else if (fp64_inner)
-            e = c.slots == 4 ? launch_chip_team<double, 4>(P, probs, c, chip_items, s)
-                             : launch_chip_team<double, 2>(P, probs, c, chip_items, s);
-        else
-            e = c.slots == 8 ? launch_chip_team<float, 8>(P, probs, c, chip_items, s)
-                             : launch_chip_team<float, 4>(P, probs, c, chip_items, s);
+    if (c.slots == 0) {
+        if (c.cw == 0) {
+            fe_kernel<<<c.count, kSolveThreads, 0, s>>>(P, probs, items + c.first);
+            return cudaGetLastError();
+        }
+        return c.cw > 1 ? launch_chip_class(fe_chip_kernel<true>, true, P, probs, c, items, s)
+                        : launch_chip_class(fe_chip_kernel<false>, false, P, probs, c, items, s);
+    }
+    if (fp64_inner)
+        return c.slots == 4 ? launch_chip_team<double, 4>(P, probs, c, items, s)
+                            : launch_chip_team<double, 2>(P, probs, c, items, s);
+    return c.slots == 8 ? launch_chip_team<float, 8>(P, probs, c, items, s)
+                        : launch_chip_team<float, 4>(P, probs, c, items, s);
+}
+
+// The on-chip launches of a plan, beside each other if `side` is given, and the global-memory one.
+cudaError_t launch_plan_solves(const SolveParams& P, const SolveParams* probs, const SolvePlan& plan,
+                               const int2* chip_items, const SolveItem* items, bool fp64_inner, cudaStream_t s,
+                               const SolveStreams* side = nullptr)
+{
+    const int launches = (int)plan.chip.size() + (plan.items.empty() ? 0 : 1);
+    const int forked = side && launches > 1 ? std::min((int)plan.chip.size(), (int)SolveStreams::kSide) : 0;
+    if (forked > 0) {
+        const cudaError_t e = cudaEventRecord(side->fork, s);
+        if (e != cudaSuccess) return e;
+    }
+    for (int k = 0; k < (int)plan.chip.size(); ++k) {
+        const cudaStream_t on = k < forked ? side->side[k] : s;
+        cudaError_t e = k < forked ? cudaStreamWaitEvent(on, side->fork, 0) : cudaSuccess;
+        if (e == cudaSuccess) e = launch_chip(P, probs, plan.chip[k], chip_items, fp64_inner, on);
+        if (e == cudaSuccess && k < forked) e = cudaEventRecord(side->join[k], on);
         if (e != cudaSuccess) return e;
     }
     const int n = (int)plan.items.size();
@@ -929,15 +943,36 @@ cudaError_t launch_plan_solves(const SolveParams& P, const SolveParams* probs, c
             else solve_items_kernel<float><<<n, kSolveThreads, 0, s>>>(P, items);
         }
     }
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    for (int k = 0; k < forked && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(s, side->join[k], 0);
+    return e;
 }
 
 }  // namespace
 
-cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const int2* chip_items,
+cudaError_t SolveStreams::create()
+{
+    cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    for (int k = 0; k < kSide && e == cudaSuccess; ++k) {
+        e = cudaStreamCreateWithFlags(&side[k], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[k], cudaEventDisableTiming);
+    }
+    return e;
+}
+
+void SolveStreams::destroy()
+{
+    if (fork) cudaEventDestroy(fork);
+    for (int k = 0; k < kSide; ++k) {
+        if (side[k]) cudaStreamDestroy(side[k]);
+        if (join[k]) cudaEventDestroy(join[k]);
+    }
+}
+
+cudaError_t launch_solve_batch(const SolveParams* probs, const SolvePlan& plan, const SolveStreams& side, const int2* chip_items,
                                const SolveItem* items, bool fp64_inner, cudaStream_t s)
 {
-    return launch_plan_solves(SolveParams{}, probs, plan, chip_items, items, fp64_inner, s);
+    return launch_plan_solves(SolveParams{}, probs, plan, chip_items, items, fp64_inner, s, &side);
 }
 
 cudaError_t launch_solve(const SolveParams& P, const SolvePlan& plan, const int2* chip_items, const SolveItem* items,
