@@ -1,5 +1,5 @@
-// Monitor preparation and Dirichlet-data scatter (grid-sized, HBM/L2-bound, negligible next
-// to the path kernel).
+// Monitor preparation, Dirichlet-data scatter and face coefficients: grid-sized, bound by memory traffic and,
+// on large grids, by the FP64 unit (each kernel's comment has its figures).
 //
 //   prep_omega_kernel : omega at every node on the current mesh at t^n (Sec. 2, Sec. 3.2),
 //                       FP64; periodic wrap nodes evaluate their canonical node so they
@@ -9,9 +9,9 @@
 //                       records in the path precision (FP64: one per node; FP32: the four
 //                       corners of every node's cell), and the previous mesh
 //                       as a displacement from the identity.
-//   scatter kernels   : the new mesh's Dirichlet data -- physical boundary (identity) and
-//                       interface estimates with periodic offsets (Sec. 3.5).
-//   face kernel       : face coefficients of the backward-Euler subdomain systems.
+//   solve_setup_kernel: the new mesh's Dirichlet data -- physical boundary (identity) and
+//                       interface estimates with periodic offsets (Sec. 3.5) -- and the face
+//                       coefficients of the backward-Euler subdomain systems.
 //
 // The prep arithmetic uses explicit round-to-nearest intrinsics (no fused multiply-add), so
 // the FP64 monitor record is reproducible independently of compiler contraction choices.

@@ -97,7 +97,12 @@ struct sdd_server {
     sdd_server_params prm{};
     cudaStream_t stream = nullptr;   // rounds: admission kernels, plan, path kernel, reduce
     cudaStream_t up = nullptr;       // host -> device uploads of admitted requests
-    cudaStream_t fin = nullptr;      // finishing requests: estimates, scatter, solves
+    // finishing requests (estimates, scatter, solves), in turn on a few streams: a request's solves are a chain of
+    // short passes on some of the SMs, and requests often finish together
+    static constexpr int kSolveStreams = 4;
+    cudaStream_t solve[kSolveStreams] = {};
+    unsigned solve_turn = 0;
+    cudaStream_t fin = nullptr;      // copies of completed requests' results
     bool fp64 = false;
     int acc_mode = kAcc64;
     int mc_grid = 1;
@@ -165,6 +170,8 @@ struct sdd_server {
         if (stream) cudaStreamSynchronize(stream);
         if (up) cudaStreamSynchronize(up);
         if (fin) cudaStreamSynchronize(fin);
+        for (cudaStream_t v : solve)
+            if (v) cudaStreamSynchronize(v);
         for (auto& kv : reqs) {
             Request* r = kv.second;
             if (r->up_ev) cudaEventDestroy(r->up_ev);
@@ -177,6 +184,8 @@ struct sdd_server {
         if (ev_b) cudaEventDestroy(ev_b);
         if (up) cudaStreamDestroy(up);
         if (fin) cudaStreamDestroy(fin);
+        for (cudaStream_t v : solve)
+            if (v) cudaStreamDestroy(v);
         for (void* v : allocs) cudaFree(v);
         for (void* v : host_allocs) cudaFreeHost(v);
     }
@@ -379,10 +388,11 @@ sdd_status finish(sdd_server* s, Request* r)
 {
     sdd_problem* p = r->p;
     const int64_t o = r->off;
+    const cudaStream_t on = s->solve[s->solve_turn++ % sdd_server::kSolveStreams];
     if (r->M > 0) {
         S_CK(launch_output(r->M, s->acc + 4 * o, s->n_done + o, s->shift + 2 * o, s->est + 2 * o, s->se + 2 * o,
-                           s->fin));
-        S_CK(launch_interp(p->interp, p->n_interp, s->est + 2 * o, s->se + 2 * o, s->fin));
+                           on));
+        S_CK(launch_interp(p->interp, p->n_interp, s->est + 2 * o, s->se + 2 * o, on));
         s->st.kernel_launches += 1 + (p->n_interp > 0 ? 1 : 0);
     }
     SolveParams S{};
@@ -395,10 +405,10 @@ sdd_status finish(sdd_server* s, Request* r)
     S.mg = p->mg; S.mg_stride = p->mg_stride;
     S.stat_iters = p->st_iters; S.stat_outer = p->st_outer; S.stat_ok = p->st_ok; S.stat_res = p->st_res;
     S_CK(launch_solve_setup(S, r->prm.periodic, r->prm.Lx, r->prm.Ly, p->nodes, r->M, s->est + 2 * o,
-                            r->prm.moving_boundary ? p->bnd64 : nullptr, s->fp64, s->fin));
-    S_CK(launch_solve(S, p->plan, p->chip_items, p->solve_items, s->fp64, s->fin));
+                            r->prm.moving_boundary ? p->bnd64 : nullptr, s->fp64, on));
+    S_CK(launch_solve(S, p->plan, p->chip_items, p->solve_items, s->fp64, on));
     s->st.kernel_launches += 1 + (int64_t)p->plan.chip.size() + (p->plan.items.empty() ? 0 : 1);
-    S_CK(cudaEventRecord(r->done_ev, s->fin));
+    S_CK(cudaEventRecord(r->done_ev, on));
     r->state = kFinishing;
     return SDD_OK;
 }
@@ -509,6 +519,8 @@ sdd_status sdd_server_create(const sdd_server_params* params, void* stream, sdd_
 #undef HALLOC
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->up, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->fin, cudaStreamNonBlocking);
+    for (cudaStream_t& v : s->solve)
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&v, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreate(&s->ev_a);
     if (e == cudaSuccess) e = cudaEventCreate(&s->ev_b);
     // idle pool nodes are never scheduled: n_done = next_total = 0; empty slot ranges

@@ -9,8 +9,8 @@
 //
 // Subdomains that fit on chip (up to about 64 x 64 unknowns in one CTA and 256 x 256 in a cluster)
 // are solved in shared memory and registers by sdd_chip.cuh.  The rest work from global memory, one
-// CTA of 512 threads per subdomain, two per SM, or a cluster of CTAs for a large one (solve_item).  Outer loop in FP64: residual b - A x of the current iterate (rims
-// included), stop when ||r||_2 <= rtol ||b||_2 for both components.  Inner solve A e = r by
+// CTA of 512 threads per subdomain, two per SM, or a cluster of CTAs for a large one (solve_item).
+// Outer loop in FP64: residual b - A x of the current iterate (rims included), stop when ||r||_2 <= rtol ||b||_2 for both components.  Inner solve A e = r by
 // conjugate gradients in the inner precision (FP32 for the FP32 modes, FP64 otherwise),
 // preconditioned by one symmetric multigrid V-cycle, then x += e (iterative refinement).
 //
