@@ -164,13 +164,14 @@ constexpr int kTasksPerRound = 256;
 // chunks of 1e4 and 1.4e4: 27.5 against 33.5), as long as a task keeps 128 substeps a lane to spread its
 // own start and reduction over.
 // The value of compensated FP32 sums depends on the grouping beyond the FP64 rounding, by about
-// 2e-8 / sqrt(n0) of the spread; they are split in the even case from 4096 paths on.
+// 2e-8 / sqrt(n0) of the spread (up to 6.5e-10 of the estimates' norm at 4096 paths); they are split in the
+// even case from 8192 paths on.
 inline int fill_task_paths(int64_t nodes, int64_t n0, int tp, bool fp64, int acc_mode, int form, int periodic,
                            int K, double dt_over_tau)
 {
     const bool even = K > 1 && (periodic || (form == 1 && dt_over_tau <= 0.01));
     if (!fp64 && !periodic && form == 0) return 0;
-    if (!fp64 && acc_mode == kAccKahan32 && !(even && n0 >= 4096)) return 0;
+    if (!fp64 && acc_mode == kAccKahan32 && !(even && n0 >= 8192)) return 0;
     const int64_t want = fp64 ? (periodic ? 1216 : 608) : 2432;
     int t = tp;
     while (t > 32 && nodes * ((n0 + t - 1) / t) < want) t >>= 1;
