@@ -362,7 +362,7 @@ sdd_status queue_mc(sdd_problem* p, int lo = 0, int hi = -1)
     PP.p_begin = p->p_begin; PP.p_count = p->p_count; PP.task_off = p->task_off;
     PP.n_active = p->n_active; PP.task_counter = p->task_counter;
     PP.task_paths = p->task_paths;
-    PP.fill = p->fill();
+    PP.fill = p->fill(p->task_paths);
     PP.task_len = p->task_len;
     ReduceParams RP{};
     RP.node_of = p->node_of; RP.p_count = p->p_count; RP.task_off = p->task_off;
@@ -1097,8 +1097,7 @@ sdd_status sdd_tune(sdd_problem* p, int32_t tune_paths_per_task, sdd_mc_config* 
             const int64_t round = n0 < (int64_t)kTasksPerRound * T ? n0 : (int64_t)kTasksPerRound * T;
             PP.task_paths = T;
             PP.task_len = p->task_len;
-            PP.fill = fill_task_paths(p->M, n0, T, p->fp64, p->acc_mode,
-                                      p->prm.form, p->prm.periodic, p->prm.substeps, p->prm.dt / p->prm.tau);
+            PP.fill = p->fill(T);
             for (int bps = 1; bps <= p->mc_max_blocks_per_sm && ce == cudaSuccess; ++bps) {
                 float ms_min = 0.f;
                 for (int rep = 0; rep < 2 && ce == cudaSuccess; ++rep) {

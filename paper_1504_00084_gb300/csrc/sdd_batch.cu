@@ -156,13 +156,22 @@ SolveParams solve_params(const sdd_problem* p)
     return S;
 }
 
-// Host copies of the per-step records (call with no step of this batch in flight).
-void refresh_records(sdd_batch* b)
+// Per-node task sizes where tasks are of tp paths.  Like the records: no upload of them may be in flight.
+void fill_task_sizes(sdd_batch* b, int tp)
 {
     for (int i = 0; i < b->n; ++i) {
         const sdd_problem* p = b->probs[i];
-        const int32_t fill = p->fill();
+        const int32_t fill = p->fill(tp);
         for (int m = 0; m < p->M; ++m) b->node_fill_host[b->node_off[i] + m] = fill;
+    }
+}
+
+// Host copies of the per-step records (call with no step of this batch in flight).
+void refresh_records(sdd_batch* b)
+{
+    fill_task_sizes(b, b->task_paths);
+    for (int i = 0; i < b->n; ++i) {
+        const sdd_problem* p = b->probs[i];
         if (b->fp64) {
             McProblem<double> R = mc_problem<double>(p);
             R.node_offset = b->node_off[i];
@@ -220,21 +229,19 @@ void set_block_size(sdd_batch* b, int tpb, int bps = 0)
     b->mc_grid = b->nsm * (b->bps > 0 ? b->bps : b->max_bps);
 }
 
-// The per-step records and per-node task sizes the round plan and the path kernel read.
 cudaError_t upload_task_sizes(sdd_batch* b)
 {
-    const size_t rec = b->fp64 ? sizeof(McProblem<double>) : sizeof(McProblem<float>);
-    cudaError_t e = cudaMemcpyAsync(b->mcprob_dev, b->mcprob_host, rec * b->n, cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess && b->M > 0)
-        e = cudaMemcpyAsync(b->node_fill, b->node_fill_host, 4 * (size_t)b->M, cudaMemcpyHostToDevice, b->stream);
-    return e;
+    if (b->M == 0) return cudaSuccess;
+    return cudaMemcpyAsync(b->node_fill, b->node_fill_host, 4 * (size_t)b->M, cudaMemcpyHostToDevice, b->stream);
 }
 
 // The launches of one step.  `capturing`: only fixed-N work (no host round trip).  first_plan:
 // stop after planning the first Monte Carlo round (used to time the path kernel).
 sdd_status record_step(sdd_batch* b, bool first_plan = false)
 {
+    const size_t rec = b->fp64 ? sizeof(McProblem<double>) : sizeof(McProblem<float>);
     int64_t launches = 0;
+    B_CK(cudaMemcpyAsync(b->mcprob_dev, b->mcprob_host, rec * b->n, cudaMemcpyHostToDevice, b->stream));
     B_CK(upload_task_sizes(b));
     B_CK(cudaMemcpyAsync(b->solve_dev, b->solve_host, sizeof(SolveParams) * b->n, cudaMemcpyHostToDevice,
                          b->stream));
@@ -649,8 +656,9 @@ sdd_status sdd_batch_tune_mc(sdd_batch* b, int32_t tune_paths_per_task, sdd_mc_c
             PP.task_paths = T;
             PP.node_fill = b->node_fill; PP.task_len = b->task_len;
             b->task_paths = T;  // read by launch_batch_mc; restored or replaced below
-            for (sdd_problem* p : b->probs) p->task_paths = T;
-            refresh_records(b);  // nothing in flight: the previous candidate's event was waited for
+            ce = cudaStreamSynchronize(b->stream);  // the uploads of the step's records, or of the last sizes
+            if (ce != cudaSuccess) break;
+            fill_task_sizes(b, T);
             ce = upload_task_sizes(b);
             for (int k = 0; k < 3 && st == SDD_OK && ce == cudaSuccess; ++k) {
                 set_block_size(b, tpbs[k]);

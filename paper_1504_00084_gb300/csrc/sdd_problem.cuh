@@ -29,10 +29,10 @@ struct sdd_problem {
     int mc_blocks_per_sm = 1;       // resident path-kernel blocks per SM (sdd_set_mc_config)
     int mc_max_blocks_per_sm = 1;   // the register limit of the path kernel
     int task_paths = sdd::kPathsPerTask;  // paths per warp task (sdd_set_mc_config)
-    // the task size that fills the GPU at this problem's size (fill_task_paths)
-    int fill() const
+    // the task size that fills the GPU at this problem's size, where tasks are of tp paths (fill_task_paths)
+    int fill(int tp) const
     {
-        return sdd::fill_task_paths(M, prm.paths_per_node, task_paths, fp64, acc_mode,
+        return sdd::fill_task_paths(M, prm.paths_per_node, tp, fp64, acc_mode,
                                     prm.form, prm.periodic, prm.substeps, prm.dt / prm.tau);
     }
     int nsm = 1;

@@ -361,7 +361,7 @@ sdd_status admit(sdd_server* s, Request* r)
     if (r->M > 0) {
         const int64_t o = r->off;
         fill_i32_kernel<<<(r->M + 255) / 256, 256, 0, s->stream>>>(s->node_prob + o, r->M, r->slot);
-        fill_i32_kernel<<<(r->M + 255) / 256, 256, 0, s->stream>>>(s->node_fill + o, r->M, p->fill());
+        fill_i32_kernel<<<(r->M + 255) / 256, 256, 0, s->stream>>>(s->node_fill + o, r->M, p->fill(p->task_paths));
         S_CK(cudaGetLastError());
         const bool adaptive = s->prm.se_target > 0;
         const int64_t n0 = s->prm.paths_per_node;

@@ -1,0 +1,60 @@
+"""Host side of the library on a CUDA runtime without a GPU (fake_cudart.cpp, preloaded): what a call queues,
+in which order it waits and which launches it chooses."""
+import ctypes
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    cxx, cuda = shutil.which("g++"), "/usr/local/cuda/include"
+    if not cxx or not os.path.isdir(cuda):
+        pytest.skip("needs g++ and the CUDA headers")
+    import __graft_entry__
+    __graft_entry__.build()
+    lib = str(tmp_path_factory.mktemp("fake") / "fake_cudart.so")
+    subprocess.run([cxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-I", cuda, os.path.join(HERE, "fake_cudart.cpp"),
+                    "-o", lib], check=True, timeout=300)
+
+    def run(name, **env):
+        r = subprocess.run([sys.executable, os.path.abspath(__file__), lib, name], cwd=ROOT, capture_output=True,
+                           text=True, timeout=300, env=dict(os.environ, LD_PRELOAD=lib, PYTHONPATH=ROOT, **env))
+        assert r.returncode == 0, (r.stdout + r.stderr)[-4000:]
+        return r.stdout
+    return run
+
+
+def problem(**kw):
+    import paper_1504_00084_gb300 as S
+    import workloads as W
+    prob = W.c0_small_fp64().replace(**kw)
+    x, y = W.identity_mesh(prob)
+    h = S.SddProblem(S.params_from(prob), x, y)
+    if prob.monitor_kind != W.MONITOR_NODAL:
+        h.set_monitor_analytic(prob.monitor_kind, prob.monitor_params)
+    return h
+
+
+def tune(lib):
+    """Every problem its own shape: records that are rewritten differ from those being uploaded."""
+    import paper_1504_00084_gb300 as S
+    hs = [problem(nx=n, ny=n, seed=n, precision=1) for n in (33, 41, 65)]
+    with S.SddBatch(hs, stream=7) as b:
+        for sizes in (False, True):
+            b.tune_mc(sizes)
+            assert lib.fake_races() == 0, "pinned records rewritten before their upload was waited for"
+
+
+def test_batch_tuning_waits_for_its_uploads(fake):
+    fake("tune")
+
+
+if __name__ == "__main__":
+    globals()[sys.argv[2]](ctypes.CDLL(sys.argv[1]))
