@@ -1248,7 +1248,8 @@ sdd_status sdd_debug_paths(sdd_problem* p, int32_t node, int64_t p_begin, int64_
 {
     if (!p) return fail(SDD_ERR_INVALID_ARG, "problem is NULL");
     if (node < 0 || node >= p->M) return fail(SDD_ERR_INVALID_ARG, "node out of range");
-    if (n_paths < 1 || p_begin < 0 || p_begin + n_paths > ((int64_t)1 << 32))
+    const int64_t end = (int64_t)1 << 32;
+    if (n_paths < 1 || p_begin < 0 || p_begin >= end || n_paths > end - p_begin)
         return fail(SDD_ERR_INVALID_ARG, "path range out of [0, 2^32)");
     const int64_t tasks = (n_paths + p->task_paths - 1) / p->task_paths;
     if (tasks > p->slot_cap) return fail(SDD_ERR_INVALID_ARG, "too many paths for one debug call");

@@ -56,5 +56,21 @@ def test_batch_tuning_waits_for_its_uploads(fake):
     fake("tune")
 
 
+def path_range(lib):
+    import paper_1504_00084_gb300 as S
+    h = problem()
+    before = lib.fake_launches()
+    for begin, n in ((1, 2 ** 63 - 1), (2 ** 32, 1), (2 ** 32 - 5, 6), (-1, 2), (0, 0), (2 ** 63 - 1, 1)):
+        assert S.lib.sdd_debug_paths(h.h, 0, begin, n, None, None, None) == S.SDD_ERR_INVALID_ARG, (begin, n)
+    assert lib.fake_launches() == before
+    h.close()
+
+
+def test_path_ranges_beyond_the_index_are_refused(fake):
+    fake("path_range")
+
+
 if __name__ == "__main__":
-    globals()[sys.argv[2]](ctypes.CDLL(sys.argv[1]))
+    LIB = ctypes.CDLL(sys.argv[1])
+    LIB.fake_launches.restype = ctypes.c_char_p
+    globals()[sys.argv[2]](LIB)
