@@ -236,10 +236,12 @@ __device__ __forceinline__ void scatter_boundary_one(int nx, int ny, double Lx, 
 // with the corner values fixed: a diagonally dominant M-matrix, by parallel cyclic reduction in shared
 // memory (each of log2 n passes joins every row with the rows 2^p away), one block a side.  A serial
 // elimination is a chain of two FP64 divisions a node: 467 us for the four sides of a 200 x 141 grid,
-// against 13.  Sides that the shared memory (`cap` nodes) does not hold are eliminated serially.
+// against 13.  Sides longer than kSideMax nodes, which the shared memory does not hold, are eliminated serially.
+// The method depends on the side's own length alone, so that a side's bits do not depend on the other sides of
+// a launch; `cap` is how many nodes the launch has shared memory for, min(its longest side, kSideMax).
 constexpr int kSideThreads = 512;
 constexpr int kSideBytes = 48;               // A, C, D twice
-constexpr int kSideMaxBytes = 200 * 1024;
+constexpr int kSideMax = 200 * 1024 / kSideBytes;
 
 template <typename T>
 __device__ __forceinline__ void boundary_side(const PrepParams& P, int s, double* sm, int cap)
@@ -531,11 +533,11 @@ __global__ void max_mean_kernel(long n, const double* v, double* out)
     }
 }
 
-// Shared memory of the boundary kernels for sides of up to n nodes (as many as it may hold).
-inline int side_cap(int n) { return n * kSideBytes <= kSideMaxBytes ? n : 0; }
+// Nodes that a launch of the boundary kernels has shared memory for, n those of its longest side.
+inline int side_cap(int n) { return n < kSideMax ? n : kSideMax; }
 cudaError_t side_allow(const void* fn)
 {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSideMaxBytes);
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSideMax * kSideBytes);
 }
 
 inline int blocks_for(long n, int threads) { return (int)((n + threads - 1) / threads); }
