@@ -27,6 +27,7 @@
 // corrections, which give the correctly rounded quotient (Markstein).  Dot products are compensated
 // FP32 pairs (exact products, 48-bit sums) instead of FP64, whose unit would need 8 us for the 16
 // thousand products of a 63 x 63 iteration; step lengths are their quotients rounded once to FP32.
+// What these see is scaled by powers of two (chip_body), so that FP32's range is enough.
 // In FP64 mode the vectors and dot products of the CG iteration are FP64, the V-cycle that
 // preconditions it FP32.
 #pragma once
@@ -49,7 +50,13 @@ template <typename TI> struct ChipSlots;
 template <> struct ChipSlots<float> { static constexpr int n = 8; };
 template <> struct ChipSlots<double> { static constexpr int n = 4; };
 
-struct ChipScalars { double stop[2]; int done; };  // what one thread works out for all
+// What one thread works out for all: the squared norm at which a component is done, the components' scale, what
+// the residual in hand has still to be multiplied with (a TI), and what comes next.
+struct ChipScalars {
+    double bn[2], goal[2], stop[2], more[2], rr[2];
+    int scale[2], target, state;
+};
+enum { kChipSolve, kChipDone, kChipAgain };
 
 // One level as a CTA holds it.  Offsets are bytes into the dynamic shared memory, alike in every CTA
 // of a cluster.
@@ -162,8 +169,8 @@ __device__ __forceinline__ bool ff_le(F2 a, F2 b) { return a.h < b.h || (a.h == 
 
 // Correctly rounded (ax, ay) / dg from inv = 1 / dg rounded: after one correction the quotient is
 // within one unit in the last place, after the second it is the rounded one (Markstein).  Exact
-// zeros stay zero; numerators below 2^-100, whose corrections would lose bits, are beyond what an
-// FP64 mesh of order 1 can show.
+// zeros stay zero; numerators below 2^-100, whose corrections would lose bits, are less than 2^-80 of
+// the residual they come from, which is scaled to 2^-20 at least.
 __device__ __forceinline__ float2 div_diag(float ax, float ay, float dg, float inv)
 {
     float qx = __fmul_rn(ax, inv), qy = __fmul_rn(ay, inv);
@@ -439,10 +446,27 @@ template <typename TI> __device__ __forceinline__ float chip_face(const void* f,
     if constexpr (sizeof(TI) == 8) return (float)f64[id];
     else return static_cast<const float*>(f)[id];
 }
-template <typename TI> __device__ __forceinline__ TI to_inner(double v)
+// 2^k, |k| <= 1022
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+// Exponent of d: -1023 for zero and subnormal numbers, 1024 for what is not finite.
+__device__ __forceinline__ int exponent(double d) { return ((__double2hiint(d) >> 20) & 0x7FF) - 1023; }
+// d 2^k as a float, rounded to nearest even, |k| <= 600: integer operations, no branch.  Below the normal range 0,
+// above it an infinity; what is not finite becomes a NaN.
+__device__ __forceinline__ float float_scaled(double d, int k)
 {
-    if constexpr (sizeof(TI) == 8) return v;
-    else return float_rn(v);
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const int E = (int)((hi >> 20) & 0x7FFu);
+    const uint64_t u = (((uint64_t)(hi + ((uint32_t)k << 20)) << 32) | lo) + 0x0FFFFFFFu + ((lo >> 29) & 1u);
+    uint32_t v = (uint32_t)(u >> 29) + 0x40000000u;
+    if ((uint32_t)(E + k) - 0x381u > 0xFCu) v = E + k < 0x381 ? 0u : 0x7F800000u;
+    if (E == 0x7FF) v = 0x7FC00000u;
+    return __uint_as_float(v | (hi & 0x80000000u));
+}
+// v 2^k
+template <typename TI> __device__ __forceinline__ TI to_inner(double v, int k)
+{
+    if constexpr (sizeof(TI) == 8) return v * pow2(k);
+    else return float_scaled(v, k);
 }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
@@ -531,16 +555,58 @@ __device__ __forceinline__ void mac(F2& a, float x, float y) { ff_mac(a, x, y); 
 __device__ __forceinline__ void mac(double& a, double x, double y) { a = fma(x, y, a); }
 __device__ __forceinline__ float ratio(F2 a, F2 b) { return b.h > 0.f ? ff_div(a, b) : 0.f; }
 __device__ __forceinline__ double ratio(double a, double b) { return b > 0.0 ? a / b : 0.0; }
-__device__ __forceinline__ double as_double(F2 a) { return (double)a.h + (double)a.l; }
-__device__ __forceinline__ double as_double(double a) { return a; }
-__device__ __forceinline__ bool is_zero(F2 a) { return a.h == 0.f; }
-__device__ __forceinline__ bool is_zero(double a) { return a == 0.0; }
 __device__ __forceinline__ F2 from_double(double t, F2) { const float h = (float)t; return F2{h, (float)(t - (double)h)}; }
 __device__ __forceinline__ double from_double(double t, double) { return t; }
 __device__ __forceinline__ bool at_most(F2 a, F2 b) { return ff_le(a, b); }
 __device__ __forceinline__ bool at_most(double a, double b) { return a <= b; }
 __device__ __forceinline__ float2 to_f2(float2 v) { return v; }
 __device__ __forceinline__ float2 to_f2(double2 v) { return make_float2((float)v.x, (float)v.y); }
+
+// d 2^k, d >= 0, by its exponent: 0 where d or the result is below the normal range
+__device__ __forceinline__ double times_pow2(double d, int k)
+{
+    const int e = exponent(d);
+    if (e == 1024) return d;
+    if (e == -1023 || e + k < -1022) return 0.0;
+    if (e + k > 1023) return INFINITY;
+    return __hiloint2double(__double2hiint(d) + (int)((uint32_t)k << 20), __double2loint(d));
+}
+// 2^k: |k| <= 60 (float), <= 1022 (double)
+template <typename TI> __device__ __forceinline__ TI pow2_of(int k)
+{
+    if constexpr (sizeof(TI) == 8) return pow2(k);
+    else return __int_as_float((127 + k) << 23);
+}
+
+// From the squared norms r0, r1 of a sweep's residual (before its scale): whether the solve is done, what the residual
+// in hand is still to be multiplied with, and where the sweep's iteration stops.  One thread: the FP64 unit would take
+// microseconds for all of them.  Not inlined, which leaves the kernel's registers to the iteration (340 -> 336 us
+// of 16 subdomains of 63 x 63).
+template <typename TI>
+__device__ __noinline__ void chip_decide(ChipScalars* scal, double r0, double r1, double rtol)
+{
+    typedef typename ChipVec<TI>::Sum Sum;
+    const double rr[2] = {r0, r1};
+    bool fine = true;
+    int state = kChipSolve;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const double goal = scal->goal[c];
+        if (goal > 1e-290) fine = fine && rr[c] <= goal;
+        else fine = fine && sqrt(scal->bn[c] > 0 ? rr[c] / scal->bn[c] : rr[c]) <= rtol;
+        const int more = rr[c] > 0.0 ? scal->target - (exponent(rr[c]) >> 1) - scal->scale[c] : 0;
+        const int k = scal->scale[c] + more;
+        if (abs(more) > 60 && scal->state != kChipAgain) state = kChipAgain;
+        *reinterpret_cast<TI*>(&scal->more[c]) = pow2_of<TI>(more);
+        scal->scale[c] = k;
+        // squared residual norm at which a component is done: half the target in FP64 (but not below 1e-14 of
+        // the start), 1e-5 of the start in FP32
+        const double st = sizeof(TI) == 8 ? fmin(0.25 * rr[c], fmax(0.25 * goal, 1e-28 * rr[c])) : 1e-10 * rr[c];
+        *reinterpret_cast<Sum*>(&scal->stop[c]) = from_double(times_pow2(st, 2 * k), Sum{});
+        scal->rr[c] = rr[c];
+    }
+    scal->state = fine ? kChipDone : state;
+}
 
 // Subdomain `sub` of the problem P by the calling CTA or cluster.
 template <typename TI, bool CL, int NS>
@@ -760,11 +826,30 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
     };
 
     int iters = 0, outer = 0, ok = 0;
-    Sum rr[2] = {none, none};  // squared residual norms
+    // A sweep's residual is taken times 2^scale, a scale for each component, so that its norm is about the root of
+    // the diagonal (by the exponents at the middle node; between 2^-20 and 2^50): squares, r.z, p.q and the cycle's
+    // values then stay in FP32's range whatever the extents and the monitor's size are.  Powers of two change no
+    // rounding.
+    if (threadIdx.x == 0) {
+        const long mid = (long)(j0 + 1 + nj / 2) * nx + (i0 + 1 + ni / 2);
+        const int most = max(exponent(dP(mid)), max(exponent(P.ce64[mid]), exponent(P.cn64[mid])));
+        scal->target = max(-20, min(50, most >> 1));
+        scal->state = kChipSolve;
+        for (int c = 0; c < 2; ++c) {
+            scal->bn[c] = bn[c];
+            scal->goal[c] = P.rtol * P.rtol * (bn[c] > 0 ? bn[c] : 1.0);
+            scal->scale[c] = scal->target - (exponent(bn[c]) >> 1);  // a guess: of the size of b
+        }
+    }
+    __syncthreads();
 #pragma unroll 1
-    for (outer = 0; outer < kMaxOuter; ++outer) {
-        // FP64 residual of the current iterate
-        rr[0] = rr[1] = none;
+    for (outer = 0; outer < kMaxOuter;) {
+        // FP64 residual of the current iterate and its squared norms; formed again (once) where the scale, that of
+        // the sweep before, is so far off that entries may have left FP32's range.  The norms are sums of FP64 squares,
+        // as the global-memory solver's: 4 of the 336 us of 16 subdomains of 63 x 63 against sums of FP32 pairs over
+        // the rounded residual, which lose what is below 1e-23 and above 1e19.
+        const int kx = scal->scale[0], ky = scal->scale[1];
+        double rr[2] = {0.0, 0.0};
 #pragma unroll
         for (int col = 0; col < 2; ++col) {
             CHIP_SLOTS(col) {
@@ -781,40 +866,35 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
                                   fma_rn(diag, P.xnew[id], -(cE * P.xnew[id + 1])))));
                 const double ay = fma_rn(-cS, P.ynew[id - nx], fma_rn(-cN, P.ynew[id + nx], fma_rn(-cW, P.ynew[id - 1],
                                   fma_rn(diag, P.ynew[id], -(cE * P.ynew[id + 1])))));
+                double rx, ry;
                 if (P.form == 0) {
-                    r[s].x = to_inner<TI>(P.xcur[id] - ax);
-                    r[s].y = to_inner<TI>(P.ycur[id] - ay);
+                    rx = P.xcur[id] - ax;
+                    ry = P.ycur[id] - ay;
                 } else {
-                    r[s].x = to_inner<TI>(fma_rn(P.om64[id], P.xcur[id], -ax));
-                    r[s].y = to_inner<TI>(fma_rn(P.om64[id], P.ycur[id], -ay));
+                    rx = fma_rn(P.om64[id], P.xcur[id], -ax);
+                    ry = fma_rn(P.om64[id], P.ycur[id], -ay);
                 }
-                mac(rr[0], r[s].x, r[s].x);
-                mac(rr[1], r[s].y, r[s].y);
+                r[s].x = to_inner<TI>(rx, kx);
+                r[s].y = to_inner<TI>(ry, ky);
+                mac(rr[0], rx, rx);
+                mac(rr[1], ry, ry);
             }
         }
-        chip_sum<CL, 2, Sum>(T, rr, red, turn);
-        // the norms' FP64 arithmetic by one thread: the unit would take microseconds for all of them
-        if (threadIdx.x == 0) {
-            bool fine = true;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const double rn = as_double(rr[c]), to = P.rtol * P.rtol * (bn[c] > 0 ? bn[c] : 1.0);
-                fine = fine && rn <= to;
-                // squared residual norm at which a component is done: half the target in FP64 (but not below
-                // 1e-14 of the start), 1e-5 of the start in FP32
-                const double st = sizeof(TI) == 8 ? fmin(0.25 * rn, fmax(0.25 * to, 1e-28 * rn)) : 1e-10 * rn;
-                *reinterpret_cast<Sum*>(&scal->stop[c]) = from_double(st, none);
-            }
-            scal->done = fine;
-        }
+        chip_sum<CL, 2, double>(T, rr, red, turn);
+        if (threadIdx.x == 0) chip_decide<TI>(scal, rr[0], rr[1], P.rtol);
         __syncthreads();
-        if (scal->done) {
+        if (scal->state == kChipAgain) continue;
+        if (scal->state == kChipDone) {
             ok = 1;
             break;
         }
         if (iters >= P.max_iter) break;
-        const Sum stop[2] = {*reinterpret_cast<const Sum*>(&scal->stop[0]), *reinterpret_cast<const Sum*>(&scal->stop[1])};
-        bool done0 = is_zero(rr[0]), done1 = is_zero(rr[1]);
+        {
+            const TI mx = *reinterpret_cast<const TI*>(&scal->more[0]), my = *reinterpret_cast<const TI*>(&scal->more[1]);
+#pragma unroll
+            for (int s = 0; s < NS; ++s) { r[s].x *= mx; r[s].y *= my; }
+        }
+        bool done0 = scal->rr[0] == 0.0, done1 = scal->rr[1] == 0.0;
         Sum rz[2] = {none, none};
 #pragma unroll
         for (int s = 0; s < NS; ++s) e[s].x = e[s].y = p[s].x = p[s].y = (TI)0;
@@ -872,8 +952,8 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
             chip_sum<CL, 4, Sum>(T, v, red, turn);  // its barrier: all are done with t, whose place p takes
             TI bx = (TI)0, by = (TI)0;
             if (!start) {
-                if (!done0 && at_most(v[2], stop[0])) done0 = true;
-                if (!done1 && at_most(v[3], stop[1])) done1 = true;
+                if (!done0 && at_most(v[2], *reinterpret_cast<const Sum*>(&scal->stop[0]))) done0 = true;
+                if (!done1 && at_most(v[3], *reinterpret_cast<const Sum*>(&scal->stop[1]))) done1 = true;
                 bx = !done0 ? ratio(v[0], rz[0]) : (TI)0;
                 by = !done1 ? ratio(v[1], rz[1]) : (TI)0;
             }
@@ -888,22 +968,25 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
                 }
             }
         }
-        // x += e
+        // x += e, the scale undone
+        const double ux = pow2(-scal->scale[0]), uy = pow2(-scal->scale[1]);
 #pragma unroll
         for (int col = 0; col < 2; ++col) {
             CHIP_SLOTS(col) {
-                P.xnew[o.id] += (double)e[s].x;
-                P.ynew[o.id] += (double)e[s].y;
+                P.xnew[o.id] = fma_rn((double)e[s].x, ux, P.xnew[o.id]);
+                P.ynew[o.id] = fma_rn((double)e[s].y, uy, P.ynew[o.id]);
             }
         }
         T.sync(1);
+        ++outer;
     }
     if (T.rank == 0 && threadIdx.x == 0) {
         P.stat_iters[sub] = iters;
         P.stat_outer[sub] = outer;
         P.stat_ok[sub] = ok;
-        const double rx = as_double(rr[0]), ry = as_double(rr[1]);
-        P.stat_res[sub] = fmax(sqrt(bn[0] > 0 ? rx / bn[0] : rx), sqrt(bn[1] > 0 ? ry / bn[1] : ry));
+        const double rx = scal->rr[0], ry = scal->rr[1];
+        const double bx = scal->bn[0], by = scal->bn[1];
+        P.stat_res[sub] = fmax(sqrt(bx > 0 ? rx / bx : rx), sqrt(by > 0 ? ry / by : ry));
     }
 #undef CHIP_SLOTS
     if constexpr (CL) cg::this_cluster().sync();  // no CTA leaves while another may still write to it
