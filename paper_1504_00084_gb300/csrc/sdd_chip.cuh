@@ -440,17 +440,11 @@ __device__ __forceinline__ void chip_sum(const Chip<CL>& T, V (&v)[NV], char* re
     }
 }
 
-// a face coefficient as the V-cycle takes it
-template <typename TI> __device__ __forceinline__ float chip_face(const void* f, const double* f64, long id)
-{
-    if constexpr (sizeof(TI) == 8) return (float)f64[id];
-    else return static_cast<const float*>(f)[id];
-}
 // 2^k, |k| <= 1022
 __device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 // Exponent of d: -1023 for zero and subnormal numbers, 1024 for what is not finite.
 __device__ __forceinline__ int exponent(double d) { return ((__double2hiint(d) >> 20) & 0x7FF) - 1023; }
-// d 2^k as a float, rounded to nearest even, |k| <= 600: integer operations, no branch.  Below the normal range 0,
+// d 2^k as a float, rounded to nearest even, |k| <= 1100: integer operations, no branch.  Below the normal range 0,
 // above it an infinity; what is not finite becomes a NaN.
 __device__ __forceinline__ float float_scaled(double d, int k)
 {
@@ -461,6 +455,24 @@ __device__ __forceinline__ float float_scaled(double d, int k)
     if ((uint32_t)(E + k) - 0x381u > 0xFCu) v = E + k < 0x381 ? 0u : 0x7F800000u;
     if (E == 0x7FF) v = 0x7FC00000u;
     return __uint_as_float(v | (hi & 0x80000000u));
+}
+// A coefficient as the V-cycle takes it.  FP32 mode: the solve's own.  FP64 mode: times 2^k, which puts those around the
+// subdomain's middle near 1 (the cycle's result is then 2^-k times as large, which the iteration does not notice),
+// and no further from it than FP32 holds over all levels; only the preconditioner sees the bounds.
+template <typename TI> __device__ __forceinline__ float chip_face(const void* f, const double* f64, long id, int k)
+{
+    if constexpr (sizeof(TI) == 8) return fminf(fmaxf(float_scaled(f64[id], k), 0x1p-100f), 0x1p100f);
+    else return static_cast<const float*>(f)[id];
+}
+template <typename TI> __device__ __forceinline__ float chip_mass(double d, int k)
+{
+    if constexpr (sizeof(TI) == 8) return fminf(float_scaled(d, k), 0x1p100f);
+    else return (float)d;
+}
+// The largest exponent of the mass and the face coefficients at node id.
+__device__ __forceinline__ int chip_exponent(const SolveParams& P, long id)
+{
+    return max(exponent(P.form == 0 ? 1.0 : P.om64[id]), max(exponent(P.ce64[id]), exponent(P.cn64[id])));
 }
 // v 2^k
 template <typename TI> __device__ __forceinline__ TI to_inner(double v, int k)
@@ -477,9 +489,12 @@ __device__ __forceinline__ double fma_rn(double a, double b, double c) { return 
 // their shared memory; a level held whole gets each CTA's part from it.
 template <typename TI, bool CL>
 __device__ __forceinline__ void chip_setup(const Chip<CL>& T, const SolveParams& P, const ChipLevel* L, int levels, int i0,
-                                           int j0)
+                                           int j0, int k)
 {
-    auto series = [](float a, float b) { return __fdiv_rn(__fmul_rn(0.5f * a, b), __fadd_rn(a, b)); };
+    auto series = [](float a, float b) {
+        const float m = __fmul_rn(0.5f * a, b), n = __fadd_rn(a, b);
+        return m >= 0x1p-100f && m <= 0x1p120f ? __fdiv_rn(m, n) : 0.5f * a * __fdiv_rn(b, n);
+    };
 #pragma unroll 1
     for (int l = 0; l < levels; ++l) {
         const ChipLevel v = L[l], u = L[l > 0 ? l - 1 : 0];
@@ -499,7 +514,7 @@ __device__ __forceinline__ void chip_setup(const Chip<CL>& T, const SolveParams&
             for (int f = T.lane; f <= v.nx; f += 32) {
                 float c;
                 if (l == 0) {
-                    c = chip_face<TI>(P.ce, P.ce64, (long)(j0 + 1 + j) * P.nx + (i0 + f));
+                    c = chip_face<TI>(P.ce, P.ce64, (long)(j0 + 1 + j) * P.nx + (i0 + f), k);
                 } else {
                     const float* fe = at<float>(T.sm, u.ce) + (2 * j + 1 - u.r0) * 2 * u.F + f;  // face 2 f of row 2 j + 1
                     c = 2 * f + 1 > u.nx ? 0.5f * fe[0] : series(fe[0], fe[u.F]);
@@ -510,7 +525,7 @@ __device__ __forceinline__ void chip_setup(const Chip<CL>& T, const SolveParams&
             for (int i = T.lane; i < v.nx; i += 32) {
                 float c;
                 if (l == 0) {
-                    c = chip_face<TI>(P.cn, P.cn64, (long)(j0 + g) * P.nx + (i0 + 1 + i));
+                    c = chip_face<TI>(P.cn, P.cn64, (long)(j0 + g) * P.nx + (i0 + 1 + i), k);
                 } else {
                     auto fine = [&](int y) {  // face row y of the level above, column 2 i + 1
                         char* from = T.sm;
@@ -535,9 +550,10 @@ __device__ __forceinline__ void chip_setup(const Chip<CL>& T, const SolveParams&
         for (int j = T.warp; j < v.nr; j += T.nw)
             for (int i = T.lane; i < v.nx; i += 32) {
                 const int o = (j * 2 + (i & 1)) * v.C + (i >> 1);
-                float d = 1.0f;
+                double w = 1.0;
                 if (P.form != 0)  // coarse node (I, J) is fine node ((I + 1) 2^l - 1, (J + 1) 2^l - 1)
-                    d = (float)P.om64[(long)(j0 + ((v.r0 + j + 1) << l)) * P.nx + (i0 + ((i + 1) << l))];
+                    w = P.om64[(long)(j0 + ((v.r0 + j + 1) << l)) * P.nx + (i0 + ((i + 1) << l))];
+                const float d = chip_mass<TI>(w, k);
                 const float dg = d + ce[(j * 2 + (i & 1)) * v.F + (i >> 1)] + ce[(j * 2 + ((i + 1) & 1)) * v.F + ((i + 1) >> 1)] +
                                  cn[o] + cn[o + 2 * v.C];
                 at<float>(T.sm, v.dg)[o] = dg;
@@ -661,7 +677,8 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
     char* red = sm + bytes;  // partial sums
     for (int k = threadIdx.x; k < bytes / 16; k += blockDim.x) reinterpret_cast<float4*>(sm)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     T.sync(1);  // rims are zero, and nobody writes to a CTA that is still clearing
-    chip_setup<TI, CL>(T, P, L, levels, i0, j0);
+    const long mid = (long)(j0 + 1 + nj / 2) * nx + (i0 + 1 + ni / 2);
+    chip_setup<TI, CL>(T, P, L, levels, i0, j0, sizeof(TI) == 8 ? -chip_exponent(P, mid) : 0);
 
     // The thread's nodes: slot s = 2 m + colour is row jl0 + m rstep, columns k0 of that colour (a row
     // wider than 64 is shared by 2^kcs warps).  A step of rows is even, so a column's parity depends on
@@ -827,13 +844,11 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
 
     int iters = 0, outer = 0, ok = 0;
     // A sweep's residual is taken times 2^scale, a scale for each component, so that its norm is about the root of
-    // the diagonal (by the exponents at the middle node; between 2^-20 and 2^50): squares, r.z, p.q and the cycle's
+    // the cycle's diagonal (by the exponents at the middle node; between 2^-20 and 2^50): squares, r.z, p.q and the cycle's
     // values then stay in FP32's range whatever the extents and the monitor's size are.  Powers of two change no
     // rounding.
     if (threadIdx.x == 0) {
-        const long mid = (long)(j0 + 1 + nj / 2) * nx + (i0 + 1 + ni / 2);
-        const int most = max(exponent(dP(mid)), max(exponent(P.ce64[mid]), exponent(P.cn64[mid])));
-        scal->target = max(-20, min(50, most >> 1));
+        scal->target = sizeof(TI) == 8 ? 0 : max(-20, min(50, chip_exponent(P, mid) >> 1));
         scal->state = kChipSolve;
         for (int c = 0; c < 2; ++c) {
             scal->bn[c] = bn[c];

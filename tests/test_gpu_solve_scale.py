@@ -47,3 +47,25 @@ def test_monitor_size_fp32(size):
     ref = _step(*size, 1, W.PREC_FP32_ACC64)
     for ew in (-40, 40):
         _same(_step(*size, 1, W.PREC_FP32_ACC64, ew=ew), ref)
+
+
+@pytest.mark.parametrize("size", SIZES)
+def test_monitor_size_fp64(size):
+    ref = _step(*size, 1, W.PREC_FP64)
+    for ew in (-300, -140, -70, 60, 130, 300):
+        _same(_step(*size, 1, W.PREC_FP64, ew=ew), ref)
+
+
+@pytest.mark.parametrize("form,e", [(0, 8), (1, 8), (1, 18)])
+def test_contrast_fp64(form, e):
+    """A monitor from 10^-e to 10^e, as far as an FP64 cycle takes the solve to its target (at form 0, the rounding
+    of an FP64 residual alone is beyond it from e = 10 on): the solve gets there."""
+    prob = W.c0_small_fp64().replace(nx=66, ny=66, px=1, py=1, form=form, precision=W.PREC_FP64, dt=1e-3,
+                                     tau=1.0 if form else 1e-2, solve_rtol=1e-8, monitor_kind=W.MONITOR_NODAL,
+                                     monitor_params=[])
+    x, y = W.identity_mesh(prob)
+    h = gpu_problem(prob, x, y, omega=10.0 ** (e * np.sin(2 * np.pi * x) * np.sin(2 * np.pi * y)))
+    _, _, status = h.step()
+    st = h.stats()
+    h.close()
+    assert status == 0 and st["solve_rel_residual"] <= prob.solve_rtol, st
