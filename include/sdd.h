@@ -236,13 +236,17 @@ sdd_status sdd_get_stats(const sdd_problem* p, sdd_stats* out);
  *   blocks_per_sm     : 1 .. max_blocks_per_sm, the register limit of the kernel (read-only
  *                       field, filled by the get calls; ignored by the set calls).
  *   paths_per_task    : 1024, 2048 (the default) or 4096.  A problem whose tasks of that size
- *                       would leave most warps idle runs finer ones of its own (a power of two,
- *                       at least 32, fixed by its parameters), compensated sums and FP32 paths of
- *                       SDD_FORM_DIV on a Dirichlet domain excepted.
+ *                       would leave most warps idle, or its last ones busy alone, runs finer ones
+ *                       of its own (a power of two, at least 32, fixed by its parameters).  Not
+ *                       FP32 paths of SDD_FORM_DIV on a Dirichlet domain; compensated sums
+ *                       (SDD_FP32_KAHAN) only from 8192 paths_per_node on, and only where paths
+ *                       rarely exit: periodic domains, or SDD_FORM_WINSLOW with dt / tau <= 0.01,
+ *                       with more than one substep.
  * What does and does not change results: threads_per_block and blocks_per_sm never do (every
  * warp runs whole tasks of fixed paths, and the sums are reduced task by task in a fixed order).
  * paths_per_task groups a node's paths differently for the estimator sums (per lane, per task,
- * per round): FP64 estimates then differ in the last bits (about 1e-16 relative per sum), and in
+ * per round): FP64 sums then differ in the last bits (about 1e-16 relative per sum), estimates from
+ * compensated sums by a few 1e-8 of their standard error, and in
  * the adaptive mode a node whose SE lies within that of the target may take another chunk.  A
  * batch uses one paths_per_task for all its problems, so a batched problem gives bitwise the
  * results of stepping it alone with the same paths_per_task.  The configuration is not part of

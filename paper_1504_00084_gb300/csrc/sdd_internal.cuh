@@ -156,16 +156,18 @@ constexpr int kTasksPerRound = 256;
 // 200 x 141 nodes, 1000 paths of about 97 substeps a node: 0.91 ms against 1.41 ms unsplit; four
 // times as many tasks win 4 % more there and cost up to 8 % where paths are shorter), in FP64 608,
 // one per SM sub-partition, whose unit a few warps fill (33 x 33, 61 x 1000 paths: 0.20 ms against
-// 0.69), twice that where no path exits (five rings, K = 1: 0.86 ms against 0.92).  FP32 paths of form 0 are the most uneven, exit after a few substeps and gain nothing
-// (sixteen bump problems in a batch: 20.3 ms against 20.6), so they keep tp.
+// 0.69), twice that where no path exits (five rings, K = 1: 0.86 ms against 0.92).  FP32 paths of form 0 are
+// the most uneven, exit after a few substeps and gain nothing, so they keep tp.
 // Periodic paths all run K substeps, and most paths of form 1 do whose diffusion over the step,
 // sqrt(2 dt / tau), is below 0.15 of the square: they leave no lane idle, and many tasks even out the
 // last wave (2032 x 4000 periodic paths, K = 100: 6.2 ms against 10.2; 1521 nodes to SE 3e-4 in
 // chunks of 1e4 and 1.4e4: 27.5 against 33.5), as long as a task keeps 128 substeps a lane to spread its
 // own start and reduction over.
-// The value of compensated FP32 sums depends on the grouping beyond the FP64 rounding, by about
-// 2e-8 / sqrt(n0) of the spread (up to 6.5e-10 of the estimates' norm at 4096 paths); they are split in the
-// even case from 8192 paths on.
+// Compensated FP32 sums round each value once more than FP64 sums do, by 2.5e-8 of it in the root mean square,
+// whatever the grouping: their estimates are off by 2.5e-8 of the standard error, and a regrouping moves them by
+// up to sqrt(2) times that, 3.6e-8 / sqrt(n0) of the paths' spread.  No accuracy is lost in finer tasks, but the
+// figures change, in the tenth digit; so those of small problems are left as whole tasks give them, and the
+// even case is split where the change is below 4e-10 of the spread, from 8192 paths a node on.
 inline int fill_task_paths(int64_t nodes, int64_t n0, int tp, bool fp64, int acc_mode, int form, int periodic,
                            int K, double dt_over_tau)
 {
