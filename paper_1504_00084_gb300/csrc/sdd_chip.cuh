@@ -1205,11 +1205,11 @@ __global__ void __launch_bounds__(kFeThreads, 1) fe_chip_kernel(const __grid_con
     fe_chip_body<CL>(sp, it.y, chip_sm);
 }
 
-// CTAs of the smallest team that holds a subdomain of ni x nj nodes (0: none of up to eight does).
-inline int fe_chip_team(int ni, int nj)
+// CTAs of the smallest team that holds a subdomain of ni x nj nodes (0: none of up to eight, or `widest`, does).
+inline int fe_chip_team(int ni, int nj, int widest)
 {
     if (ni <= 0 || nj <= 0) return 1;
-    for (int cw = 1; cw <= 8; cw *= 2)
+    for (int cw = 1; cw <= 8 && cw <= widest; cw *= 2)
         if (nj >= cw && (int64_t)((nj + cw - 1) / cw) * ni <= kFeThreads * kFeSlots && ni <= 4096 &&
             fe_chip_bytes(ni, nj, cw) <= kChipSmem)
             return cw;
@@ -1218,10 +1218,10 @@ inline int fe_chip_team(int ni, int nj)
 
 // Team of a subdomain of ni x nj interior nodes: CTAs (0: it does not fit), warps per CTA, slots of
 // its kernel, dynamic shared memory.  The fewest CTAs that hold it -- a cluster barrier costs about a
-// microsecond, ten times a CTA's -- as a function of the size alone, so that a subdomain gives the
-// same bits in every launch.  Warps: the fewest, from four, with half the slots, so that small
+// microsecond, ten times a CTA's -- as a function of the size (and of the widest cluster that the device takes)
+// alone, so that a subdomain gives the same bits in every launch.  Warps: the fewest, from four, with half the slots, so that small
 // subdomains share an SM and run the smaller kernel.
-inline void chip_team(int ni, int nj, bool fp64, ChipLaunch* c)
+inline void chip_team(int ni, int nj, bool fp64, int widest, ChipLaunch* c)
 {
     c->cw = c->nw = c->slots = c->smem = 0;
     const int most = fp64 ? ChipSlots<double>::n : ChipSlots<float>::n;
@@ -1230,7 +1230,7 @@ inline void chip_team(int ni, int nj, bool fp64, ChipLaunch* c)
         return;
     }
     if (ni > 512 || nj > 4096) return;
-    for (int cw = 1; cw <= kChipWidth; cw *= 2) {
+    for (int cw = 1; cw <= widest; cw *= 2) {
         if (cw > 1 && nj < 2 * cw) return;
         ChipLevel L[kChipLevels];
         int levels = 0, p_off = 0;

@@ -28,6 +28,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <map>
 #include <mutex>
 #include <set>
 
@@ -792,8 +793,13 @@ void solve_subs(int prob, int nx, int ny, int px, int py, int scheme, std::vecto
     }
 }
 
+namespace {
+int widest_cluster(bool fp64);
+}
+
 SolvePlan solve_plan(std::vector<SolveSub> subs, bool fp64)
 {
+    const int widest = widest_cluster(fp64);
     // longest first; ties in the given order
     std::stable_sort(subs.begin(), subs.end(), [](const SolveSub& a, const SolveSub& c) {
         return (int64_t)a.ni * a.nj > (int64_t)c.ni * c.nj;
@@ -808,16 +814,16 @@ SolvePlan solve_plan(std::vector<SolveSub> subs, bool fp64)
     for (const SolveSub& v : subs) {
         ChipLaunch c{};
         if (v.scheme == 1) {
-            c.cw = fe_chip_team(v.ni, v.nj);
+            c.cw = fe_chip_team(v.ni, v.nj, widest);
             if (c.cw > 0 && v.ni > 0 && v.nj > 0) {
-                while (c.cw < 8 && 2 * c.cw * n_fe <= kSms && v.nj >= 6 * c.cw) c.cw *= 2;
+                while (2 * c.cw <= std::min(8, widest) && 2 * c.cw * n_fe <= kSms && v.nj >= 6 * c.cw) c.cw *= 2;
                 c.smem = fe_chip_bytes(v.ni, v.nj, c.cw);
             } else if (c.cw > 0) {
                 c.smem = 1024;
             }
             c.nw = kFeThreads / 32;
         } else {
-            chip_team(v.ni, v.nj, fp64, &c);
+            chip_team(v.ni, v.nj, fp64, widest, &c);
         }
         if (c.cw > 0 || v.scheme == 1) {
             size_t k = 0;
@@ -870,21 +876,60 @@ cudaError_t chip_allow(const void* fn, bool cluster)
 
 typedef void (*ChipKernel)(const SolveParams, const SolveParams*, const int2*);
 
+// A launch of `count` clusters of cw CTAs.
+void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int cw, int count, int threads, int smem)
+{
+    cfg.gridDim = dim3((unsigned)(cw * count));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cw;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+}
+
+// CTAs of the widest cluster of the solve kernels that the current device takes (1 to kChipWidth): a GPU with a
+// share of its SMs may have no place for 16, and a launch of them would fail.  Asked once per device.
+int widest_cluster(bool fp64)
+{
+    static std::mutex mu;
+    static std::map<std::pair<int, bool>, int> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find({dev, fp64});
+    if (it != known.end()) return it->second;
+    const ChipKernel kernels[3] = {fp64 ? chip_kernel<double, true, 4> : chip_kernel<float, true, 8>,
+                                   fp64 ? chip_kernel<double, true, 2> : chip_kernel<float, true, 4>, fe_chip_kernel<true>};
+    int widest = 1;
+    for (int cw = 2; cw <= kChipWidth; cw *= 2) {
+        bool fits = true;
+        for (int k = 0; k < (cw <= 8 ? 3 : 2) && fits; ++k) {
+            const void* fn = reinterpret_cast<const void*>(kernels[k]);
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute at[1];
+            cluster_config(cfg, at, cw, 1, 512, kChipSmem);
+            int n = 0;
+            fits = chip_allow(fn, true) == cudaSuccess && cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0;
+        }
+        if (!fits) break;
+        widest = cw;
+    }
+    cudaGetLastError();
+    known[{dev, fp64}] = widest;
+    return widest;
+}
+
 cudaError_t launch_chip_class(ChipKernel fn, bool cluster, const SolveParams& P, const SolveParams* probs,
                               const ChipLaunch& c, const int2* items, cudaStream_t s)
 {
     cudaError_t e = chip_allow(reinterpret_cast<const void*>(fn), cluster);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(c.cw * c.count));
-    cfg.blockDim = dim3((unsigned)(32 * c.nw));
-    cfg.dynamicSmemBytes = (size_t)c.smem;
-    cfg.stream = s;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)c.cw;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
+    cluster_config(cfg, at, c.cw, c.count, 32 * c.nw, c.smem);
+    cfg.stream = s;
     cfg.numAttrs = cluster ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, fn, P, probs, items + c.first);
 }

@@ -70,6 +70,34 @@ def test_path_ranges_beyond_the_index_are_refused(fake):
     fake("path_range")
 
 
+def clusters(lib):
+    """Solves whose team would be wider than the device's widest cluster go to narrower teams or to global memory."""
+    import paper_1504_00084_gb300 as S
+    widest = int(os.environ["FAKE_CLUSTER"])
+    for kw in (dict(nx=258, ny=258), dict(nx=130, ny=129), dict(nx=120, ny=120, subdomain_scheme=1),
+               dict(nx=66, ny=66, subdomain_scheme=1), dict(nx=33, ny=33)):
+        for precision in (0, 1):
+            before = len(lib.fake_launches())
+            with problem(px=1, py=1, precision=precision, **kw) as h:
+                try:
+                    h.step()
+                except S.SddError:  # nothing ran: no solve has reported convergence
+                    pass
+            made = [line.rsplit(" ", 4) for line in lib.fake_launches()[before:].decode().splitlines()]
+            solves = [m for m in made if "chip_kernel" in m[0] or "items_kernel" in m[0] or "fe_kernel" in m[0]]
+            assert len(solves) == 1 and int(solves[0][4]) <= widest, (kw, made)
+            on_chip = "chip_kernel" in solves[0][0]
+            if kw["nx"] == 33 or (widest == 16 and precision == 1):  # in FP64 256 x 256 fits nowhere
+                assert on_chip, (kw, made)
+            if kw["nx"] == 258 and widest < 16:
+                assert not on_chip, (kw, made)
+
+
+@pytest.mark.parametrize("widest", [1, 2, 4, 8, 16])
+def test_teams_fit_the_device(fake, widest):
+    fake("clusters", FAKE_CLUSTER=str(widest))
+
+
 if __name__ == "__main__":
     LIB = ctypes.CDLL(sys.argv[1])
     LIB.fake_launches.restype = ctypes.c_char_p
