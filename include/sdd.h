@@ -347,8 +347,9 @@ int64_t sdd_debug_bounds_violations(void);
  * Many problems of uneven grid and subdomain counts advance one alternating step together
  * (Sec. 3.6 for each): per problem the monitor preparation and the scatter of Dirichlet data;
  * ONE persistent path-kernel launch per round for the interface nodes of all problems, and
- * ONE launch for all subdomain solves (one CTA per (problem, subdomain)).  Each problem's
- * results are bitwise those of sdd_step on it alone (own seed, local node ids in the Philox
+ * the subdomain solves of all problems in one launch per size class (one CTA or a cluster of up
+ * to 16 per (problem, subdomain)), the classes beside each other on streams of the batch.  Each
+ * problem's results are bitwise those of sdd_step on it alone (own seed, local node ids in the Philox
  * counter, per-node path schedule, fixed-order reductions).  All problems must share
  * precision, se_target and paths_per_node (and max_paths_per_node when adaptive), and their
  * interface nodes must number below 2^23 in total (else SDD_ERR_INVALID_ARG); the batch
@@ -403,7 +404,7 @@ void sdd_batch_destroy(sdd_batch* b);
  * the path kernel: a round is ONE persistent path-kernel launch over the interface nodes of all
  * running requests (a shared node pool in which each request holds a contiguous range), and a
  * request whose nodes have all reached the service level is finished at once (estimates,
- * Dirichlet scatter, subdomain solves, on a second stream) while the others keep sampling.
+ * Dirichlet scatter, subdomain solves, on other streams) while the others keep sampling.
  * A request's result is bitwise that of sdd_step on a problem created alone with the same
  * parameters, mesh, monitor and step index (own seed, local node ids in the Philox counter,
  * per-node path schedule, fixed-order reductions).

@@ -3,8 +3,8 @@
 // Many mesh problems of uneven grid and subdomain counts advance one alternating step
 // together: per problem, the monitor preparation and the Dirichlet-data scatter; then ONE
 // persistent path-kernel launch per round serves the interface nodes of every problem (the
-// round plan runs over the concatenated node list, every task carries its problem), and ONE
-// launch solves every subdomain of every problem (one CTA per (problem, subdomain)).
+// round plan runs over the concatenated node list, every task carries its problem), and the
+// subdomains of all problems are solved in one launch per size class, a CTA or a cluster each.
 //
 // A problem's results do not depend on its batch: its paths use its own seed and local node
 // ids in the Philox counter, its nodes follow their own chunk schedule, and every sum is a

@@ -54,22 +54,8 @@ __host__ __device__ __forceinline__ U4 philox4x32_10(U4 c, uint32_t k0, uint32_t
     return c;
 }
 
-// The same generator with its ten round keys given: rk[2r], rk[2r + 1] is the key of round r
-// (key0 + r W0, key1 + r W1).  A launch over one problem reads them from its parameter block,
-// so no key arithmetic runs per call.
-__device__ __forceinline__ U4 philox4x32_10_rk(U4 c, const uint32_t* rk)
-{
-    constexpr uint32_t kM0 = 0xD2511F53u, kM1 = 0xCD9E8D57u;
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t h0 = __umulhi(kM0, c.x), l0 = kM0 * c.x;
-        const uint32_t h1 = __umulhi(kM1, c.z), l1 = kM1 * c.z;
-        c = U4{h1 ^ c.y ^ rk[2 * r], l1, h0 ^ c.w ^ rk[2 * r + 1], l0};
-    }
-    return c;
-}
-
-// Round keys of philox4x32_10_rk for the 64-bit seed (key0 = low word, key1 = high word).
+// The generator's ten round keys for the 64-bit seed (key0 = low word, key1 = high word): rk[2r], rk[2r + 1] is the
+// key of round r (key0 + r W0, key1 + r W1).  The path kernel reads them from its parameter block.
 inline void philox_round_keys(uint64_t seed, uint32_t rk[20])
 {
     uint32_t k0 = (uint32_t)(seed & 0xFFFFFFFFu), k1 = (uint32_t)(seed >> 32);
@@ -258,7 +244,6 @@ struct PlanParams {
     int64_t* task_off;
     int32_t* n_active;
     int32_t* task_counter;
-    int32_t* host_n_active;    // mapped pinned host word
     // optional planning order: M positions taken from n_ranges pool ranges in list order
     const int32_t* range_off;  // first node of each range (null: positions are node ids)
     const int32_t* range_pre;  // exclusive prefix of the range lengths (n_ranges + 1)

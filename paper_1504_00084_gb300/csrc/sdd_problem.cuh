@@ -101,7 +101,7 @@ struct sdd_problem {
     struct Out { void* dst; const void* from; size_t bytes; };
     std::vector<Out> staged, late;  // copies to the caller: from the staging, or made after the status is known
     std::vector<char> v_stats;      // the solves' records when they have no pinned place
-    int mc_lo = 0, mc_hi = 0, mc_timed = 0;  // of the Monte Carlo that is queued
+    int mc_timed = 0;               // timed path-kernel launches of the Monte Carlo that is queued
     cudaEvent_t count_ev[sdd::kRoundsAhead + 1] = {};  // after the copies of the round counts
     sdd_stats stats{};
     std::vector<void*> allocs;

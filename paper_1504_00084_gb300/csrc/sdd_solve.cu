@@ -242,13 +242,6 @@ __device__ __forceinline__ void mg_first_sweep(const Team<CW>& tm, const MgLevel
     tm.sync();
 }
 
-template <typename TI, int CW>
-__device__ __forceinline__ void mg_zero(const Team<CW>& tm, const MgLevel<TI>& L)
-{
-    for (int k = tm.tid(); k < L.nx * L.ny; k += tm.nthreads()) L.x[k] = Pair<TI>{(TI)0, (TI)0};
-    tm.sync();
-}
-
 // b_{l+1} = full weighting of the residual t_l = b_l - A_l x_l
 template <typename TI, int CW>
 __device__ __forceinline__ void mg_restrict(const Team<CW>& tm, const MgLevel<TI>& F, const MgLevel<TI>& C)
