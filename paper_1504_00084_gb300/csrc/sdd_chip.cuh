@@ -414,7 +414,8 @@ __device__ __forceinline__ void chip_gather(V (&v)[NV], const V* part, int n, in
 #pragma unroll
     for (int p = 0; p < NV; ++p) v[p] = SumOf<V>::from(t, p * group);
 }
-template <bool CL, int NV, typename V>
+// WARP0: the totals in the first warp alone (an FP64 addition costs an SM 16 clocks a warp).
+template <bool CL, int NV, typename V, bool WARP0 = false>
 __device__ __forceinline__ void chip_sum(const Chip<CL>& T, V (&v)[NV], char* red, int& turn)
 {
     // without a cluster the warps' totals alternate instead
@@ -434,9 +435,9 @@ __device__ __forceinline__ void chip_sum(const Chip<CL>& T, V (&v)[NV], char* re
             }
         }
         T.sync(1);
-        chip_gather<NV>(v, team, T.cw, T.lane);
+        if (!WARP0 || T.warp == 0) chip_gather<NV>(v, team, T.cw, T.lane);
     } else {
-        chip_gather<NV>(v, part, T.nw, T.lane);
+        if (!WARP0 || T.warp == 0) chip_gather<NV>(v, part, T.nw, T.lane);
     }
 }
 
@@ -597,7 +598,7 @@ template <typename TI> __device__ __forceinline__ TI pow2_of(int k)
 // From the squared norms r0, r1 of a sweep's residual (before its scale): whether the solve is done, what the residual
 // in hand is still to be multiplied with, and where the sweep's iteration stops.  One thread: the FP64 unit would take
 // microseconds for all of them.  Not inlined, which leaves the kernel's registers to the iteration (340 -> 336 us
-// of 16 subdomains of 63 x 63).
+// of 16 subdomains of 63 x 63; 334 with the norms' totals in one warp).
 template <typename TI>
 __device__ __noinline__ void chip_decide(ChipScalars* scal, double r0, double r1, double rtol)
 {
@@ -861,7 +862,7 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
     for (outer = 0; outer < kMaxOuter;) {
         // FP64 residual of the current iterate and its squared norms; formed again (once) where the scale, that of
         // the sweep before, is so far off that entries may have left FP32's range.  The norms are sums of FP64 squares,
-        // as the global-memory solver's: 4 of the 336 us of 16 subdomains of 63 x 63 against sums of FP32 pairs over
+        // as the global-memory solver's: 4 of the 334 us of 16 subdomains of 63 x 63 against sums of FP32 pairs over
         // the rounded residual, which lose what is below 1e-23 and above 1e19.
         const int kx = scal->scale[0], ky = scal->scale[1];
         double rr[2] = {0.0, 0.0};
@@ -895,7 +896,7 @@ __device__ __forceinline__ void chip_body(const SolveParams& P, int sub, ChipLev
                 mac(rr[1], ry, ry);
             }
         }
-        chip_sum<CL, 2, double>(T, rr, red, turn);
+        chip_sum<CL, 2, double, true>(T, rr, red, turn);
         if (threadIdx.x == 0) chip_decide<TI>(scal, rr[0], rr[1], P.rtol);
         __syncthreads();
         if (scal->state == kChipAgain) continue;
