@@ -322,7 +322,8 @@ sdd_status sdd_get_monitor(sdd_problem* p, double* omega, double* w_xi, double* 
 /* Test hook: per-path records of paths p_begin .. p_begin + n_paths - 1 of interface node
  * `node`, computed by the same kernel code as sdd_interface_mc: val_xy (n x 2 doubles),
  * exit_step (substeps taken), exit_side (0: xi=0, 1: xi=1, 2: eta=0, 3: eta=1, 4: none).
- * Any output may be NULL.  Uses the current monitor and mesh; does not change state. */
+ * Any output may be NULL.  Uses the current monitor and mesh; does not change state.
+ * p_begin >= 0, n_paths >= 1, p_begin + n_paths <= 2^32. */
 sdd_status sdd_debug_paths(sdd_problem* p, int32_t node, int64_t p_begin, int64_t n_paths,
                            double* val_xy, int32_t* exit_step, int8_t* exit_side);
 
