@@ -1059,8 +1059,8 @@ __device__ __forceinline__ void fe_chip_body(const SolveParams& P, int sub, char
     const int i0 = split_line(I, nx, P.px), i1 = split_line(I + 1, nx, P.px);
     const int j0 = split_line(J, P.ny, P.py), j1 = split_line(J + 1, P.ny, P.py);
     const int ni = i1 - i0 - 1, nj = j1 - j0 - 1;
-    if (ni <= 0 || nj <= 0) {  // no interior (a team of one CTA)
-        if (tid == 0) {
+    if (ni <= 0 || nj <= 0) {  // no interior
+        if (T.rank == 0 && tid == 0) {
             P.stat_iters[sub] = 1; P.stat_outer[sub] = 0; P.stat_ok[sub] = 1; P.stat_res[sub] = 0.0;
         }
         return;

@@ -98,6 +98,25 @@ def test_teams_fit_the_device(fake, widest):
     fake("clusters", FAKE_CLUSTER=str(widest))
 
 
+def euler_launches(lib):
+    """Forward-Euler subdomains of uneven sizes (some without an interior) that can all run at once are one launch:
+    launches of a problem follow each other, each a chain of substeps."""
+    import paper_1504_00084_gb300 as S
+    for nx, ny, px, py in ((66, 35, 6, 5), (4, 40, 2, 6), (7, 26, 5, 2), (41, 120, 1, 7), (33, 33, 2, 2), (9, 9, 8, 8)):
+        before = len(lib.fake_launches())
+        with problem(nx=nx, ny=ny, px=px, py=py, subdomain_scheme=1) as h:
+            try:
+                h.step()
+            except S.SddError:  # nothing ran: no solve has reported convergence
+                pass
+        made = [line for line in lib.fake_launches()[before:].decode().splitlines() if "fe_" in line]
+        assert len(made) == 1, ((nx, ny, px, py), made)
+
+
+def test_uneven_forward_euler_is_one_launch(fake):
+    fake("euler_launches")
+
+
 if __name__ == "__main__":
     LIB = ctypes.CDLL(sys.argv[1])
     LIB.fake_launches.restype = ctypes.c_char_p
