@@ -804,8 +804,7 @@ SolvePlan solve_plan(std::vector<SolveSub> subs, bool fp64)
     // forward Euler: its results do not depend on the team, so few subdomains get more CTAs each, as
     // long as all run at once and every CTA has a few rows.  Where one team does for all and all run at once, they
     // get the same, and with it one launch: two sizes of team are two chains of substeps one after the
-    // other (30 subdomains of 10 x 5 and 10 x 6, 48 substeps:
-    // 278 us in two launches, 137 in one)
+    // other (30 subdomains of 10 x 5 and 10 x 6, 48 substeps: 278 us in two launches, 137 in one)
     int64_t n_fe = 0;
     int fe_team = 1, least = INT_MAX;
     for (const SolveSub& v : subs) {
@@ -905,7 +904,10 @@ int widest_cluster(bool fp64)
     static std::mutex mu;
     static std::map<std::pair<int, bool>, int> known;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
     std::lock_guard<std::mutex> lock(mu);
     const auto it = known.find({dev, fp64});
     if (it != known.end()) return it->second;
